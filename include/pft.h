@@ -22,7 +22,11 @@
  *   - PFT_SCFT_REAL: fields are real float64 arrays W+ (= i*omega+) and W- (= omega-);
  *     PFT_CL_COMPLEX: fields are complex128 arrays omega+ and omega- (interleaved
  *     re, im).  All API-facing arrays are float64 / complex128 in either precision.
- *   - PFT_FP64 runs every step in double.  PFT_FP32_MIXED runs the propagators, FFTs
+ *   - PFT_FP64 runs every step to double accuracy: fields, propagators, Boltzmann factors and
+ *     sums are doubles; the pencil march's convolutions along axes of 16, 32, 48, 64, 96 and
+ *     128 points are exact sums of integer products on the tensor cores (values scaled by
+ *     the largest of their line, 2^-55 of it the rounding), rounded once to double.
+ *     PFT_FP32_MIXED runs the propagators, FFTs
  *     and Boltzmann factors in float (the integrand q*qd of the contour quadrature is
  *     the float product of the two float propagators) and keeps the field update, the
  *     contour quadrature sums, every spatial reduction, Q, lnQ and H in double.

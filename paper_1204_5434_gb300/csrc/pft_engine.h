@@ -188,12 +188,23 @@ struct SeppGeom {
   int n[3];
   int kind;
   int lv = 0;  // line variant: 1 = register lines (FP32, x and y lengths with a register plan)
+  int* err = nullptr;  // error word of bounded waits
 };
 // Launch j (0..Ns) of a separable pencil march for `members` entries starting at ss (for
 // j >= 1 the entries of contour step j; j = 0 uses those of step 1).  Real fields need
 // ny and nz even.  Returns cudaErrorInvalidValue for a length without an FFT plan.
 cudaError_t sepp_launch_f32(const SeppGeom& g, const BatchStep* ss, int j, int members, cudaStream_t sm);
 cudaError_t sepp_launch_f64(const SeppGeom& g, const BatchStep* ss, int j, int members, cudaStream_t sm);
+// One convolution launch of the FP64 march on the tensor cores (pft_tc64.cuh): axis ax with the
+// Boltzmann products of its kernel (ax 0: x B_s, store, x B_{s+1}; ax 1: none; ax 2: pw 1 the
+// march's first launch, pw 2 as ax 0).  Lengths of 16, 32, 48, 64, 96 and 128 points, where it is
+// the faster of the two at every size (above that X does not fit tensor memory; other lengths are
+// no multiple of the product's 16).  The axis' table (tc64_axis_table of its factors at k = 0 ..
+// n/2) lies behind the factors d[ax], at the next multiple of 256 bytes.
+bool tc64_axis_applies(const SeppGeom& g, int ax);
+cudaError_t tc_launch_f64(const SeppGeom& g, const BatchStep* ss, int ax, int pw, int members, cudaStream_t sm);
+size_t tc64_axis_table_bytes(int n);
+void tc64_axis_table(int n, const long double* d, unsigned char* dst);
 // the same march in double-float arithmetic (FP64 history, dd tables and factors)
 cudaError_t sepp_launch_dd(const SeppGeom& g, const BatchStep* ss, int j, int members, cudaStream_t sm);
 

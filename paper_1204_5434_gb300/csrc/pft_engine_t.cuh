@@ -125,6 +125,8 @@ class EngineT : public Engine {
     for (int a = 0; a < 3; a++) {
       c.sd_off[a] = off;
       off = al(off + sizeof(T) * (size_t)c.n[a]);
+      // behind them the axis' table of the tensor-core convolution (pft_tc64.cuh)
+      if (std::is_same<T, double>::value) off = al(off + tc64_axis_table_bytes(c.n[a]));
     }
     // FP64 twiddles of the full x, y, z lengths (the transforms of the semi-implicit step)
     for (int a = 0; a < 3; a++) {
@@ -176,6 +178,22 @@ class EngineT : public Engine {
         const int mm = (m <= na / 2) ? m : m - na;
         const double k = 2.0 * M_PI * (double)mm / c.L[a];
         sd[m] = (T)(exp(-k * k * c.ds) / (double)na);
+      }
+      // the axis' table of the tensor-core convolution; an axis like an earlier one shares its values
+      const size_t tcb = std::is_same<T, double>::value ? tc64_axis_table_bytes(na) : 0;
+      unsigned char* tct = h.data() + c.sd_off[a] + al(sizeof(T) * (size_t)na);
+      int like = -1;
+      for (int b = 0; b < a; b++)
+        if (c.n[b] == na && c.L[b] == c.L[a]) like = b;
+      if (tcb && like >= 0) {
+        memcpy(tct, h.data() + c.sd_off[like] + al(sizeof(T) * (size_t)na), tcb);
+      } else if (tcb) {
+        std::vector<long double> da((size_t)na / 2 + 1);
+        for (int m = 0; m <= na / 2; m++) {
+          const long double k = 2.0L * 3.14159265358979323846264338327950288L * m / (long double)c.L[a];
+          da[m] = expl(-k * k / (long double)c.Ns);
+        }
+        tc64_axis_table(na, da.data(), tct);
       }
     }
     return cudaMemcpyAsync(c.tables, h.data(), off, cudaMemcpyHostToDevice, c.stream);
@@ -396,6 +414,7 @@ class EngineT : public Engine {
     for (int a = 0; a < 3; a++) g.n[a] = c.n[a];
     g.kind = (c.kind == PFT_SCFT_REAL) ? 0 : 1;
     g.lv = (c.plan_plane == 3) ? c.plan_xv : 0;
+    g.err = c.kerr;
     const BatchStep* st = (const BatchStep*)c.stepsCK;
     const BatchStep* cst = st + c.ckRoff.back();
     const QuadPair* pr = (const QuadPair*)c.pairsCK;
@@ -743,6 +762,7 @@ class EngineT : public Engine {
     for (int a = 0; a < 3; a++) g.n[a] = c.n[a];
     g.kind = (c.kind == PFT_SCFT_REAL) ? 0 : 1;
     g.lv = (c.plan_plane == 3) ? c.plan_xv : 0;
+    g.err = c.kerr;
     for (int j = 0; j <= c.Ns; j++) {
       if (members == 2) mark(c, KK_PAIR_STEP);
       const BatchStep* ss = st + (size_t)2 * (j == 0 ? 0 : j - 1);
@@ -1176,6 +1196,7 @@ class EngineT : public Engine {
     for (int a = 0; a < 3; a++) sg.n[a] = g.n[a];
     sg.kind = (g.kind == PFT_SCFT_REAL) ? 0 : 1;
     sg.lv = ((plan & 15) == 3) ? plan >> 4 : 0;
+    sg.err = err;
     return std::is_same<T, float>::value ? sepp_launch_f32(sg, ss, j, nact, sm) : sepp_launch_f64(sg, ss, j, nact, sm);
   }
 

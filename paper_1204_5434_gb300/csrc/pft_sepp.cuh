@@ -492,14 +492,28 @@ cudaError_t sepp_launch_k(const SeppGeom& g, const BatchStep* ss, int j, int mem
   const long long nx = g.n[0], ny = g.n[1], nz = g.n[2];
   const long long nzz = KIND == 0 ? nz / 2 : nz;  // complex elements per row
   cudaError_t e = cudaSuccess;
+  if constexpr (std::is_same<T, double>::value) {  // convolutions on the tensor cores where they apply
+    const int ax = (j & 1) ? 0 : 2;
+    if (j == 0 && tc64_axis_applies(g, 2)) return tc_launch_f64(g, ss, 2, 1, members, sm);
+    if (j > 0) {
+      if (tc64_axis_applies(g, 1)) {
+        e = tc_launch_f64(g, ss, 1, 0, members, sm);
+      } else {
+        PFT_SEPP_AXIS(g.n[1], e = (sepp_line_n<T, N, KIND, 0, 1>(ss, nx * nzz, nzz, ny * nzz, nzz, members, sm, g.lv)));
+      }
+      if (e != cudaSuccess) return e;
+      if (tc64_axis_applies(g, ax)) return tc_launch_f64(g, ss, ax, 2, members, sm);
+    }
+  } else if (j > 0) {
+    // Ky on the lines (x, z element) along y
+    PFT_SEPP_AXIS(g.n[1], e = (sepp_line_n<T, N, KIND, 0, 1>(ss, nx * nzz, nzz, ny * nzz, nzz, members, sm, g.lv)));
+    if (e != cudaSuccess) return e;
+  }
   if (j == 0) {  // x B_1, Kz
     const long long nl = KIND == 0 ? nx * ny / 2 : nx * ny;
     PFT_SEPP_AXIS(g.n[2], e = (sepp_z_n<T, N, KIND, 1>(ss, nl, members, sm)));
     return e;
   }
-  // Ky on the lines (x, z element) along y
-  PFT_SEPP_AXIS(g.n[1], e = (sepp_line_n<T, N, KIND, 0, 1>(ss, nx * nzz, nzz, ny * nzz, nzz, members, sm, g.lv)));
-  if (e != cudaSuccess) return e;
   if (j & 1) {  // Kx, x B_j, store q_j, x B_{j+1}, Kx
     PFT_SEPP_AXIS(g.n[0], e = (sepp_line_n<T, N, KIND, 2, 0>(ss, ny * nzz, ny * nzz, 0, ny * nzz, members, sm, g.lv)));
   } else {      // Kz, x B_j, store q_j, x B_{j+1}, Kz

@@ -1,0 +1,556 @@
+// pft_tc64.cuh -- the FP64 convolutions of the separable march on the tensor cores
+// (pft_tcgen05.cuh): tiles of 128 lines times the circulant matrix of the axis.
+//
+// Both factors carry FP64 accuracy as sums of small integers, every one exact in FP16, because
+// GB300 does 2 FP64 multiply-adds a cycle and SM and 4096 FP16 ones on the tensor core.
+//   X: line by line scaled to 2^54 / S with S the power of two above the line's largest value,
+//      rounded to an integer and cut into six digits of 9 bits, X = sum_i X_i 2^(9 (5 - i)),
+//      |X_0| <= 2^9, |X_i| <= 2^8: the rounding is 2^-55 of S, below an FP64 rounding of the
+//      largest value.
+//   K: kern 2^p = sum_j K_j 2^(-9 j), j = 0..6, |K_j| < 2^11 (K_0: sum |K_0| <= 2^13).  The
+//      rounding of every K_j is chosen so that the sum of K_0 is 2^p and the sum of every other
+//      K_j is zero: what the products left out below do to the mean of a line vanishes.
+// Level l collects the products X_i K_j with i + j = l in one FP32 accumulator of the tensor
+// core: integers below 2^24 in sum, hence exact in any order of addition.  Levels 0 to 5 (21
+// products) are added up in 64-bit integers, level 5 with X_0 K_6 (K_6 stored 2^-9 smaller: an
+// error of the kernel acts at every step, and its seventh digit keeps that below 1e-18 a step);
+// the other products of level 6 are 2^-57 of S.  The sum is rounded once, to FP64.  Propagator slices against the FP64 oracle: 2e-16 to 8e-16 relative
+// (the FFT pair in FP64: the same or larger; the products with the Boltzmann factors set it).
+//
+// One CTA holds one tile: G warpgroups of 128 threads (thread = line) and one more warp that
+// issues the products, level by level into a ring of NB accumulators, while the warpgroups
+// read the levels before.  A line with an infinity or a NaN becomes NaN, as under the FFT.
+//
+// What bounds it: at 64 points a tile takes 15,000 cycles without and 37,000 with the
+// Boltzmann products -- 3,900 for the products of a convolution (2,700 at the tensor core's
+// rate), 4,400 for the digits and 4,200 for the conversion back, both at the integer pipe's 64
+// operations a cycle and SM, and 8,200 for the two FP64 multiplications by B.  The FFT pair
+// needs about 26 FP64 operations a point and convolution, 13 cycles an SM; this 1.8 to 4.
+// Measured, both marches of one solve, Ns = 100, FFT pair -> this: 32^3 real 3.68 -> 1.88 ms,
+// 64^3 real 6.50 -> 3.29, 64^3 complex 12.0 -> 4.83, 128^3 real 50.5 -> 13.5, 128^3 complex
+// 102.9 -> 37.2.
+#pragma once
+#include "pft_tcgen05.cuh"
+
+namespace pft {
+
+template <int N> struct Tc64Cfg {
+  static constexpr int NS = 6;  // digits
+  static constexpr int PPT = N <= 64 ? 16 : 32;
+  static constexpr int G = N / PPT;
+  static constexpr int WORK = 128 * G;
+  static constexpr int THREADS = WORK + 32;
+  static constexpr int CW = N <= 96 ? N : 64;
+  static constexpr int NCH = N / CW;
+  static constexpr int CPW = CW / PPT;
+  static constexpr int NB = N <= 64 ? 4 : 2;
+  static constexpr int COLS_USED = NS * N / 2 + NB * CW;
+  static constexpr int COLS = COLS_USED <= 128 ? 128 : (COLS_USED <= 256 ? 256 : 512);
+  static constexpr int NSLOT = 2 * (N / 8) - 1;
+  static constexpr int TAB = 16 + (NS + 1) * NSLOT * 128;
+  static_assert(N % PPT == 0 && N % CW == 0 && CW % PPT == 0 && COLS_USED <= 512, "whole chunks in tensor memory");
+};
+inline bool tc64_axis_ok(int n) { return n == 16 || n == 32 || n == 48 || n == 64 || n == 96 || n == 128; }
+inline size_t tc64_table_bytes(int n) { return 16 + (size_t)7 * (2 * (n / 8) - 1) * 128; }
+
+// Host arithmetic of the table: the unevaluated sum of two doubles (Knuth's TwoSum, FMA product),
+// the same on every host whatever its long double is.
+struct Dd64 {
+  double h, l;
+};
+inline Dd64 dd64_sum(double a, double b) {
+  const double s = a + b, t = s - a;
+  return {s, (a - (s - t)) + (b - t)};
+}
+inline Dd64 dd64_add(Dd64 a, Dd64 b) {
+  const Dd64 s = dd64_sum(a.h, b.h);
+  return dd64_sum(s.h, s.l + (a.l + b.l));
+}
+inline Dd64 dd64_mul(Dd64 a, Dd64 b) {
+  const double p = a.h * b.h;
+  return dd64_sum(p, fma(a.h, b.h, -p) + (a.h * b.l + a.l * b.h));
+}
+inline Dd64 dd64_from(long double x) {
+  const double h = (double)x;
+  return {h, (double)(x - (long double)h)};
+}
+
+// The table of one axis: the header {int p}, then the blocks of K_0 .. K_6: block s
+// of a digit holds kern[(8 (s - n/8 + 1) + r - e) mod n] at row r, element e.  d: the axis' factors exp(-k_a^2 ds) at k = 0 .. n/2.
+inline void tc64_build_table(int n, const long double* d, unsigned char* dst) {
+  const int h = n / 2;
+  std::vector<Dd64> cs((size_t)n), r((size_t)h + 1);
+  for (int j = 0; j <= h; j++) {
+    cs[j] = dd64_from(cosl(2.0L * 3.14159265358979323846264338327950288L * j / n));
+    if (j) cs[n - j] = cs[j];
+  }
+  double kmax = 0.0, ksum = 0.0;
+  auto mult = [&](int j) { return (j && j < n - j) ? 2 : 1; };
+  for (int j = 0; j <= h; j++) {
+    Dd64 a = {0.0, 0.0};
+    for (int k = 0; k <= h; k++) {
+      const Dd64 f = dd64_from(d[k] * (mult(k) / (long double)n));
+      a = dd64_add(a, dd64_mul(f, cs[(size_t)((j * k) % n)]));
+    }
+    r[j] = a;
+    kmax = std::max(kmax, fabs(a.h));
+    ksum += mult(j) * fabs(a.h);
+  }
+  // |K_0| <= 2^11 - 2 (exact in FP16 after the correction of its sum), sum |K_0| <= 2^13
+  int p = 13;
+  while (p > 0 && (kmax * ldexp(1.0, p) > 2046.0 || ksum * ldexp(1.0, p) > 8192.0 + 1e-3)) p--;
+  for (int j = 0; j <= h; j++) r[j] = {ldexp(r[j].h, p), ldexp(r[j].l, p)};
+  memset(dst, 0, 16);
+  memcpy(dst, &p, sizeof(p));
+  const int nslot = 2 * (n / 8) - 1;
+  std::vector<double> q((size_t)h + 1);
+  std::vector<__half> q16((size_t)3 * n);  // the digit at distance j, over three periods
+  __half* out = reinterpret_cast<__half*>(dst + 16);
+  for (int sl = 0; sl < 7; sl++) {
+    long long sum = 0;
+    for (int j = 0; j <= h; j++) {
+      q[j] = rint(r[j].h);
+      sum += mult(j) * (long long)q[j];
+    }
+    long long off = (sl == 0 ? (1LL << p) : 0LL) - sum;  // to be added to the digits
+    while (off != 0) {  // the value whose rounding went furthest the other way takes a unit
+      const int dir = off > 0 ? 1 : -1;
+      const bool odd = (off & 1) != 0;
+      int b = -1;
+      double best = -1e300;
+      for (int j = 0; j <= h; j++) {
+        if (odd != (mult(j) == 1)) continue;
+        const double gain = dir * ((r[j].h - q[j]) + r[j].l);
+        if (gain > best) {
+          best = gain;
+          b = j;
+        }
+      }
+      q[b] += dir;
+      off -= (long long)dir * mult(b);
+    }
+    for (int j = 0; j < n; j++) {
+      const __half v = __float2half_rn((float)(q[j <= h ? j : n - j] * (sl == 6 ? 1.0 / 512.0 : 1.0)));
+      q16[j] = q16[j + n] = q16[j + 2 * n] = v;
+    }
+    for (int b = 0; b < nslot; b++)
+      for (int row = 0; row < 8; row++)
+        for (int e = 0; e < 8; e++) *out++ = q16[(size_t)(n + 8 * (b - n / 8 + 1) + row - e)];
+    for (int j = 0; j <= h; j++) {  // exact: the remainders of a rounding, times 2^9
+      const Dd64 t = dd64_sum(r[j].h - q[j], r[j].l);
+      r[j] = {t.h * 512.0, t.l * 512.0};
+    }
+  }
+}
+
+// z lines: staging rows of a warp, 16 bytes of padding a row
+template <int N, int KIND> struct Tc64Z {
+  static constexpr int PPT = Tc64Cfg<N>::PPT;
+  static constexpr int PITCH = KIND ? 2 * PPT + 2 : PPT + 2;  // doubles
+  static constexpr int ROWS = KIND ? 16 : 32;
+  static constexpr int WARP_DOUBLES = ROWS * PITCH;
+  static constexpr size_t BYTES = (size_t)(Tc64Cfg<N>::WORK / 32) * WARP_DOUBLES * sizeof(double);
+};
+template <int N, int KIND, int PW, int AX> constexpr size_t tc64_smem() {
+  return tc_align(Tc64Cfg<N>::TAB) + Tc64Cfg<N>::WORK * sizeof(int) + 128 +
+         (AX == 2 ? Tc64Z<N, KIND>::BYTES : (PW == 2 ? (size_t)N * 128 * sizeof(double) : 0));
+}
+
+// The tensor-core sum t as FP64, t 2^(eb - 1085) rounded to nearest, on the integer pipe (the
+// FP64 pipe converts 2 a cycle and SM): normalised by a shift, rounded by adding the bit below
+// the last one kept (the carry runs into the exponent).  eb keeps the exponent in range.
+__device__ __forceinline__ double tc64_to_double(long long t, int eb) {
+  const unsigned long long a = (unsigned long long)(t < 0 ? -t : t);
+  const bool small = (unsigned)(a >> 32) == 0u;
+  const unsigned h = small ? (unsigned)a : (unsigned)(a >> 32), l = small ? 0u : (unsigned)a;
+  const int lz = __clz((int)h);
+  const unsigned hn = __funnelshift_l(l, h, lz), ln = l << (lz & 31);
+  const unsigned L = __funnelshift_r(ln, hn, 11);
+  const unsigned H = (hn >> 11) + ((unsigned)(eb - lz - (small ? 32 : 0)) << 20);
+  const unsigned long long r = (((unsigned long long)H << 32) | L) + ((ln >> 10) & 1u);
+  const unsigned top = (h == 0u ? 0u : (unsigned)(r >> 32)) | ((unsigned)((unsigned long long)t >> 32) & 0x80000000u);
+  return __hiloint2double((int)top, (int)(unsigned)r);
+}
+// FP64 in the digits' form: X, the integer nearest x in units of 2^(eL - 1076) (eL the biased
+// exponent of the line's largest value, at least kTc64MinExp), plus the digits' biases, above 8
+// bits of no meaning: digit i of X plus its bias is at bit 8 + 9 (5 - i).  The biases, 256 (512
+// for the leading digit), make all digits non-negative.  Ties go to even: values of a few bits
+// below the unit meet them half of the time, and a fixed direction would shift every step's mean.
+constexpr int kTc64MinExp = 80;  // a line below 2^-943 counts as 2^-943
+__device__ __forceinline__ unsigned long long tc64_digits(double x, int eL) {
+  constexpr unsigned long long BIAS =
+      256ull * (1ull + (1ull << 9) + (1ull << 18) + (1ull << 27) + (1ull << 36)) + (512ull << 45);
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int sh = eL + 2 - (int)((hi >> 20) & 0x7ffu);  // 2 and more; a zero or subnormal: 64 and more
+  const unsigned mh = __funnelshift_l(lo, (hi & 0xfffffu) | 0x100000u, 11), ml = lo << 11;  // leading bit 63
+  const bool far = sh >= 32;
+  const unsigned a = far ? mh : ml, b = far ? 0u : mh;
+  const int s5 = far ? sh - 32 : sh;
+  const unsigned wl = __funnelshift_rc(a, b, s5), wh = s5 >= 32 ? 0u : b >> s5;
+  const unsigned sg = (unsigned)((int)hi >> 31);
+  const unsigned long long v = (((unsigned long long)(wh ^ sg) << 32) | (wl ^ sg)) - (((unsigned long long)sg << 32) | sg);
+  return v + ((BIAS << 8) + 127ull) + (((unsigned)v >> 8) & 1u);
+}
+
+// AX 0, 1: lines along x or y; line c of the nlines starts at (c / cin) s_outer + c % cin doubles
+// and its points lie s_k apart (complex fields: real and imaginary parts are lines of their own,
+// in neighbouring threads).  AX 2: lines along z, nlines rows of N points (complex fields: two
+// rows a pencil), staged in shared memory warp by warp.
+// PW 0: the convolution; PW 1: x B_1 on q_0 = st.in, convolution; PW 2: convolution, x B_s,
+// store q_s, then (if st.Bnext) x B_{s+1}, convolution.
+template <int N, int KIND, int PW, int AX>
+__global__ void __launch_bounds__(Tc64Cfg<N>::THREADS, 1)
+kb_tc64_line(const BatchStep* __restrict__ st, int nlines, int cin, int s_outer, int s_k, int* err) {
+  using CF = Tc64Cfg<N>;
+  constexpr int G = CF::G, PPT = CF::PPT, CW = CF::CW, NCH = CF::NCH, CPW = CF::CPW, NB = CF::NB, NS = CF::NS;
+  constexpr uint32_t DCOL = NS * N / 2;  // first accumulator column
+  const BatchStep& s = st[blockIdx.y];
+  extern __shared__ __align__(16) unsigned char smraw[];
+  int* lexp = reinterpret_cast<int*>(smraw + tc_align(CF::TAB));
+  uint64_t* full = reinterpret_cast<uint64_t*>(lexp + CF::WORK);
+  uint64_t* empty = full + NCH * NB;  // full: one set a chunk, so that its readers meet every phase
+  uint64_t* done = empty + NB;
+  uint32_t* tbase = reinterpret_cast<uint32_t*>(done + 1);
+  static_assert(NCH == 1 || NS % NB == 0, "a chunk's levels use every accumulator equally often");
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform
+  const bool more = PW == 2 && s.Bnext != nullptr;
+
+  // ---- table, barriers, tensor memory
+  {
+    const uint4* t4 = reinterpret_cast<const uint4*>(reinterpret_cast<const char*>(s.d[AX]) + tc_align(N * sizeof(double)));
+    uint4* d4 = reinterpret_cast<uint4*>(smraw);
+    for (int i = tid; i < CF::TAB / 16; i += CF::THREADS) d4[i] = t4[i];
+  }
+  if (tid == 0) {
+#pragma unroll
+    for (int i = 0; i < NCH * NB; i++) mbar_init(full + i, 1);
+#pragma unroll
+    for (int i = 0; i < NB; i++) mbar_init(empty + i, 4 * CPW);
+    mbar_init(done, 1);
+    mbar_init_fence();
+  }
+  if (warp == 4 * G) tc_alloc(tbase, CF::COLS);
+  fence_proxy_async_smem();
+  constexpr int NJ = NCH * NS;  // jobs a turn: (chunk, level) in order, job t in accumulator t % NB
+
+  if (warp == 4 * G) {
+    // ================================================= the issuing warp
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tm = __shfl_sync(0xffffffffu, *tbase, 0);
+    const uint64_t k0 = tc_desc(smem_addr(smraw) + 16);
+    for (int turn = 0; turn < (more ? 2 : 1); turn++) {
+      named_sync(1, CF::THREADS);  // X is in tensor memory
+      tc_fence_after();
+      for (int ch = 0; ch < NCH; ch++) {
+        for (int l = 0; l < NS; l++) {
+          const int t = ch * NS + l, b = t % NB;
+          if (t >= NB) {  // job t - NB has been read: it was use t / NB - 1 of this turn's
+            mbar_wait(empty + b, (unsigned)(turn * ((NJ - b + NB - 1) / NB) + t / NB - 1) & 1u, err, 1);
+            tc_fence_after();
+          }
+          __syncwarp();
+          if (elect_one()) {
+            const uint32_t d = tm + DCOL + (uint32_t)(b * CW);
+            const int np = l + 1 + (l == NS - 1 ? 1 : 0);
+            for (int i = 0; i < np; i++) {  // X_i K_{l-i}, and X_0 K_6 with the last level
+              const int xi = i > l ? 0 : i, kj = i > l ? NS : l - i;
+              const uint32_t a = tm + (uint32_t)(xi * (N / 2));
+              const uint64_t kd = k0 + (uint64_t)((kj * CF::NSLOT + ch * (CW / 8)) * 8);
+#pragma unroll
+              for (int j = 0; j < N / 16; j++)
+                tc_mma_f16_ts(d, a + 8 * j, kd + (N / 8 - 2 - 2 * j) * 8, tc_idesc(CW), (i > 0 || j > 0) ? 1u : 0u);
+            }
+            tc_commit(full + ch * NB + b);
+            if (t == NJ - 1) tc_commit(done);
+          }
+          __syncwarp();
+        }
+      }
+    }
+    __syncthreads();  // every accumulator has been read
+    tc_fence_after();
+    tc_dealloc(tm, CF::COLS);
+    return;
+  }
+
+  // =================================================== the lines' warpgroups
+
+  const int g = warp >> 2, m = tid & 127;
+  const int col = blockIdx.x * 128 + m;
+  const bool valid = col < nlines;
+  const int colc = valid ? col : 0;
+  double* F = reinterpret_cast<double*>(s.spec);
+  const double* B = reinterpret_cast<const double*>(s.B);
+  const double* Bn = reinterpret_cast<const double*>(s.Bnext);
+  int base, step;
+  if (AX != 2) {
+    base = (colc / cin) * s_outer + (colc % cin) + g * PPT * s_k;
+    step = s_k;
+  } else if (KIND == 0) {
+    base = colc * N + g * PPT;
+    step = 1;
+  } else {
+    base = (colc >> 1) * (2 * N) + 2 * g * PPT + (colc & 1);
+    step = 2;
+  }
+  using ZS = Tc64Z<N, KIND>;
+  double* area = reinterpret_cast<double*>(smraw + tc_align(CF::TAB) + CF::WORK * sizeof(int) + 128);
+  double* zs = area + (AX == 2 ? warp * ZS::WARP_DOUBLES : 0);
+  const int row0 = blockIdx.x * 128 + (m & ~31);
+  double* zrow = KIND ? zs + (lane >> 1) * ZS::PITCH + (lane & 1) : zs + lane * ZS::PITCH;
+  // rows of the warp into and out of shared memory in 16-byte pieces
+  constexpr int CPR = KIND ? PPT : PPT / 2;
+  auto zglob = [&](int r, int c2) -> long long {  // offset of piece c2 of row r
+    return KIND ? ((long long)(row0 >> 1) + r) * (2 * N) + 2 * (g * PPT + c2)
+                : (long long)(row0 + r) * N + g * PPT + 2 * c2;
+  };
+  auto zin = [&](const double* src) {
+#pragma unroll 4
+    for (int i = lane; i < ZS::ROWS * CPR; i += 32) {
+      const int r = i / CPR, c2 = i % CPR;
+      if (row0 + (KIND ? 2 * r : r) < nlines)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(zs + r * ZS::PITCH + 2 * c2)),
+                     "l"(src + zglob(r, c2))
+                     : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  auto zwait = [&]() {
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncwarp();
+  };
+  auto zout = [&](double* dst) {
+    __syncwarp();
+#pragma unroll 4
+    for (int i = lane; i < ZS::ROWS * CPR; i += 32) {
+      const int r = i / CPR, c2 = i % CPR;
+      if (row0 + (KIND ? 2 * r : r) < nlines)
+        *reinterpret_cast<double2*>(dst + zglob(r, c2)) = *reinterpret_cast<const double2*>(zs + r * ZS::PITCH + 2 * c2);
+    }
+    __syncwarp();
+  };
+  auto zat = [&](int i) -> double& { return zrow[KIND ? 2 * i : i]; };
+  auto mulB = [&](double x, double b) -> double {
+    if constexpr (KIND == 0) {
+      return x * b;
+    } else {
+      const double bo = __shfl_xor_sync(0xffffffffu, b, 1), xo = __shfl_xor_sync(0xffffffffu, x, 1);
+      return (lane & 1) ? x * bo + xo * b : x * b - xo * bo;
+    }
+  };
+
+  double v[PPT];
+  if constexpr (AX == 2) {
+    zin(PW == 1 ? reinterpret_cast<const double*>(s.in) : F);
+    zwait();
+#pragma unroll
+    for (int i = 0; i < PPT; i++) v[i] = valid ? zat(i) : 0.0;
+    if constexpr (PW == 1) {
+      __syncwarp();
+      zin(B);
+      zwait();
+#pragma unroll
+      for (int i = 0; i < PPT; i++) v[i] = mulB(v[i], valid ? zat(i) : 0.0);
+      __syncwarp();
+    }
+  } else {
+    const double* fp = F + base;
+#pragma unroll
+    for (int i = 0; i < PPT; i++) {
+      v[i] = *fp;
+      fp += step;
+    }
+    if constexpr (PW == 2) {  // B_s of the tile, rows of 128 consecutive doubles
+      for (int i = tid; i < N * 64; i += CF::WORK) {
+        const int r = i >> 6, c2 = (i & 63) * 2;
+        if ((int)blockIdx.x * 128 + c2 < nlines)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(area + r * 128 + c2)),
+                       "l"(B + (long long)r * s_k + blockIdx.x * 128 + c2)
+                       : "memory");
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tm = __shfl_sync(0xffffffffu, *tbase, 0);
+  const uint32_t tlane = tm + ((uint32_t)(warp & 3) << 21);
+  const int p = *reinterpret_cast<const int*>(smraw);
+  const int ch = g / CPW;       // this warpgroup's chunk
+  // how often before: the chunk's barrier full[ch][l % NB] at its level l
+  auto full_use = [](int turn, int l) -> unsigned {
+    return (unsigned)(turn * ((NS - l % NB + NB - 1) / NB) + l / NB);
+  };
+  int ebase = 0;
+  bool odd = false;
+  double sc1 = 1.0, sc2 = 1.0;
+
+  auto split = [&](int turn) {
+    unsigned mx = 0;
+#pragma unroll
+    for (int i = 0; i < PPT; i++) mx = max(mx, (unsigned)__double2hiint(v[i]) & 0x7fffffffu);
+    lexp[g * 128 + m] = (int)(mx >> 20);
+    if (turn) {  // every product of the convolution before has read X
+      mbar_wait(done, 0, err, 1);
+      tc_fence_after();
+    }
+    named_sync(2, CF::WORK);
+    int eL = 0;
+#pragma unroll
+    for (int w = 0; w < G; w++) eL = max(eL, lexp[w * 128 + m]);
+    odd = eL < 300 || eL > 1900;
+    const bool bad = eL == 0x7ff;  // an infinity or a NaN: the line becomes NaN
+    eL = max(eL, kTc64MinExp);
+    const int eC = odd ? 1000 : eL;  // results near either end of the range: scaled in two parts
+    ebase = eC - 47 - p + 62;
+    if (odd) {
+      const int d = eL - 1000;  // -920 .. 1046
+      sc1 = __hiloint2double((1023 + d / 2) << 20, 0);
+      sc2 = bad ? __hiloint2double(0x7fffffff, -1) : __hiloint2double((1023 + d - d / 2) << 20, 0);
+    }
+#pragma unroll
+    for (int j = 0; j < PPT / 8; j++) {
+      unsigned lo[8], hi[8];
+#pragma unroll
+      for (int i = 0; i < 8; i++) {
+        const unsigned long long y = tc64_digits(v[8 * j + i], eL);
+        lo[i] = (unsigned)y;
+        hi[i] = (unsigned)(y >> 32);
+      }
+#pragma unroll
+      for (int dgt = 0; dgt < NS; dgt++) {  // digit 0 is the leading one
+        uint32_t w[4];
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+          auto dig = [&](int q) -> unsigned {
+            switch (dgt) {
+              case 5: return lo[q] >> 8;
+              case 4: return lo[q] >> 17;
+              case 3: return __funnelshift_r(lo[q], hi[q], 26);
+              case 2: return hi[q] >> 3;
+              case 1: return hi[q] >> 12;
+              default: return hi[q] >> 21;
+            }
+          };
+          const unsigned pk = __byte_perm(dig(2 * i), dig(2 * i + 1), 0x5410);
+          // FP16 1024 + digit by its bits, then exactly minus (1024 + bias)
+          const unsigned hb = dgt == 0 ? (pk & 0x07ff07ffu) + 0x64006400u : ((pk & 0x01ff01ffu) | 0x64006400u);
+          const __half2 hv = __hsub2(*reinterpret_cast<const __half2*>(&hb),
+                                     __half2half2(__ushort_as_half(dgt == 0 ? 0x6600 : 0x6500)));
+          w[i] = *reinterpret_cast<const uint32_t*>(&hv);
+        }
+        // the two halves of each 16 points swapped
+        tc_st4(tlane + (uint32_t)(dgt * (N / 2) + g * (PPT / 2) + 4 * (j ^ 1)), w);
+      }
+    }
+    tc_wait_st();
+    tc_fence_before();
+    asm volatile("bar.arrive 1, %0;" ::"r"(CF::THREADS) : "memory");
+  };
+
+  const uint32_t dacc = tlane + DCOL + (uint32_t)((g % CPW) * PPT);
+  long long acc[PPT];
+  // the levels of this warpgroup's chunk, added up in units of 2^-39 of level 0's
+  auto collect = [&](int turn) {
+#pragma unroll
+    for (int l = 0; l < NS; l++) {
+      const int b = l % NB;  // the accumulator of job ch NS + l of this turn
+      mbar_wait(full + ch * NB + b, full_use(turn, l) & 1u, err, 1);
+      tc_fence_after();
+#pragma unroll
+      for (int j = 0; j < PPT / 8; j++) {
+        uint32_t r[8];
+        tc_ld8(dacc + (uint32_t)(b * CW) + 8 * j, r);
+        tc_wait_ld();
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+          const int d = __float2int_rn(__uint_as_float(r[i]));
+          long long& a = acc[8 * j + i];
+          if (l == 0) a = (long long)((unsigned long long)(unsigned)(d << 7) << 32);
+          else if (l == 5) a += (d + 32) >> 6;
+          else a += (long long)d * (l == 1 ? (1 << 30) : (l == 2 ? (1 << 21) : (l == 3 ? (1 << 12) : (1 << 3))));
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(empty + b)) : "memory");
+    }
+  };
+  // the convolution's values into v: unit 2^(eL + 1 - 1023) 2^-9 2^-p 2^-39
+  auto finish = [&]() {
+#pragma unroll
+    for (int k = 0; k < PPT; k++) v[k] = tc64_to_double(acc[k], ebase);
+    if (odd) {
+#pragma unroll 1
+      for (int k = 0; k < PPT; k += 8) {
+#pragma unroll
+        for (int i = 0; i < PPT; i++)
+          if (i / 8 == k / 8) v[i] = v[i] * sc1 * sc2;
+      }
+    }
+  };
+
+  split(0);
+  if constexpr (PW == 2) {
+    const bool same = (Bn == B);
+    double* q = reinterpret_cast<double*>(s.out);
+    if constexpr (AX == 2) {
+      __syncwarp();
+      zin(B);
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      named_sync(2, CF::WORK);  // every thread's pieces of the tile have landed
+    }
+    collect(0);
+    if constexpr (AX == 2) zwait();
+    finish();
+    const double* bt = area + (g * PPT) * 128 + m;
+    double* qp = q + base;
+#pragma unroll
+    for (int k = 0; k < PPT; k++) {
+      double bk;
+      if constexpr (AX == 2) bk = valid ? zat(k) : 0.0;
+      else bk = bt[k * 128];
+      const double x = mulB(v[k], bk);
+      if constexpr (AX == 2) zat(k) = x;
+      else if (valid) *qp = x;
+      qp += step;
+      v[k] = same ? mulB(x, bk) : x;
+    }
+    if constexpr (AX == 2) zout(q);
+    if (more) {
+      if (!same) {
+        const double* bp = Bn + base;
+#pragma unroll
+        for (int k = 0; k < PPT; k++) {
+          v[k] = mulB(v[k], valid ? *bp : 0.0);
+          bp += step;
+        }
+      }
+      split(1);
+      collect(1);
+    }
+  } else {
+    collect(0);
+  }
+  if (PW != 2 || more) {
+    double* fo = F + base;
+    finish();
+#pragma unroll
+    for (int k = 0; k < PPT; k++) {
+      if constexpr (AX == 2) zat(k) = v[k];
+      else if (valid) *fo = v[k];
+      fo += step;
+    }
+    if constexpr (AX == 2) zout(F);
+  }
+  tc_fence_before();
+  __syncthreads();
+}
+
+}  // namespace pft

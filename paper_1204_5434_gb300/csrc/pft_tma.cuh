@@ -51,12 +51,15 @@ __device__ __forceinline__ bool mbar_test(uint64_t* bar, unsigned parity) {
 }
 
 // Bounded wait for the phase with parity `parity`.  On expiry sets *err (if given) to
-// `code` and returns false.
+// `code` and returns false; a wait longer than a millisecond also gives up once another
+// wait has set *err, so that a kernel of many waits ends soon after its first expiry.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity, int* err, int code) {
   if (mbar_test(bar, parity)) return true;
   const unsigned long long t0 = global_ns();
   while (!mbar_test(bar, parity)) {
-    if (global_ns() - t0 > kWaitNs) {
+    const unsigned long long dt = global_ns() - t0;
+    if (dt > 1000000ull && err && *(volatile int*)err != 0) return false;
+    if (dt > kWaitNs) {
       if (err) atomicExch(err, code);
       return false;
     }
