@@ -105,6 +105,8 @@ struct CtxData {
   size_t ddB_off[2] = {0, 0};
   void* stepsD = nullptr;   // [2 * Ns]
   void* stepsg = nullptr;   // [2 * Ns] BatchStep: the two spectra of the box derivative
+  void* gspec = nullptr;    // [gsteps][2][Ms] spectra of a group of its steps (null: spec and spec2, one step)
+  int gsteps = 1;
   // checkpointed history (ckK >= 2) on the separable pencil march: the step entries of the
   // forward march [Ns], of every segment recompute [<= Ns] and of the conjugate march [Ns];
   // the quadrature pairs (q_{Ns-m}, qd_m) [Ns]; K conjugate slices of the current chunk
