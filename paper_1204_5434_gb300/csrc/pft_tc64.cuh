@@ -21,37 +21,48 @@
 // issues the products, level by level into a ring of NB accumulators, while the warpgroups
 // read the levels before.  A line with an infinity or a NaN becomes NaN, as under the FFT.
 //
-// What bounds it: at 64 points a tile takes 15,000 cycles without and 37,000 with the
-// Boltzmann products -- 3,900 for the products of a convolution (2,700 at the tensor core's
-// rate), 4,400 for the digits and 4,200 for the conversion back, both at the integer pipe's 64
-// operations a cycle and SM, and 8,200 for the two FP64 multiplications by B.  The FFT pair
-// needs about 26 FP64 operations a point and convolution, 13 cycles an SM; this 1.8 to 4.
-// Measured, both marches of one solve, Ns = 100, FFT pair -> this: 32^3 real 3.68 -> 1.88 ms,
-// 64^3 real 6.50 -> 3.29, 64^3 complex 12.0 -> 4.83, 128^3 real 50.5 -> 13.5, 128^3 complex
-// 102.9 -> 37.2.
+// What bounds it: the integer pipe (64 operations a cycle and SM; ncu: busy throughout) beside the
+// products.  A 64-point tile of 128 lines takes 10,500 cycles without and 25,700 with the Boltzmann
+// products: 3,800 for the products of a convolution (2,800 at the tensor core's rate), 2,200 for the
+// digits, 7,100 for the two factors and q in FP64, 2,000 each to load and to store.  With FP64
+// fields (FX 0) 15,000 and 37,000: 4,400 for the digits, 4,200 for each conversion back, 8,200 for
+// two FP64 multiplications by B.  The FFT pair needs about 26 FP64 operations a point and
+// convolution, 13 cycles an SM, this 1.3 to 3.
+// Measured, both marches of one solve, Ns = 100, FFT pair -> FX 0 -> FX 1 (ms): 32^3 real 3.68 ->
+// 1.88 -> 1.49, 64^3 real 6.50 -> 3.29 -> 2.64, 64^3 complex 12.0 -> 4.83 -> 2.99, 128^3 real 50.5 ->
+// 13.5 -> 9.93, 128^3 complex 102.9 -> 37.2 -> 23.7.
+// Tried: skipping the k steps where a digit of the kernel is zero (128 points: 26,000 -> 29,000
+// cycles, the branches cost more than a quarter of the products); the smallest level first (saves
+// two operations a point, but its eight products delay the first reading: 3,800 -> 5,100 cycles);
+// a reading warpgroup's warp issuing the products (3,800 -> 4,700).
 #pragma once
+#include <type_traits>
+
 #include "pft_tcgen05.cuh"
 
 namespace pft {
 
+constexpr int kTc64Head = 16;  // bytes of a table's header
+// outputs a product computes: the axis, at 128 points half of it
+constexpr int tc64_chunk(int n) { return n <= 96 ? n : 64; }
 template <int N> struct Tc64Cfg {
   static constexpr int NS = 6;  // digits
   static constexpr int PPT = N <= 64 ? 16 : 32;
   static constexpr int G = N / PPT;
   static constexpr int WORK = 128 * G;
   static constexpr int THREADS = WORK + 32;
-  static constexpr int CW = N <= 96 ? N : 64;
+  static constexpr int CW = tc64_chunk(N);
   static constexpr int NCH = N / CW;
   static constexpr int CPW = CW / PPT;
   static constexpr int NB = N <= 64 ? 4 : 2;
   static constexpr int COLS_USED = NS * N / 2 + NB * CW;
   static constexpr int COLS = COLS_USED <= 128 ? 128 : (COLS_USED <= 256 ? 256 : 512);
   static constexpr int NSLOT = 2 * (N / 8) - 1;
-  static constexpr int TAB = 16 + (NS + 1) * NSLOT * 128;
+  static constexpr int TAB = kTc64Head + (NS + 1) * NSLOT * 128;
   static_assert(N % PPT == 0 && N % CW == 0 && CW % PPT == 0 && COLS_USED <= 512, "whole chunks in tensor memory");
 };
 inline bool tc64_axis_ok(int n) { return n == 16 || n == 32 || n == 48 || n == 64 || n == 96 || n == 128; }
-inline size_t tc64_table_bytes(int n) { return 16 + (size_t)7 * (2 * (n / 8) - 1) * 128; }
+inline size_t tc64_table_bytes(int n) { return kTc64Head + (size_t)7 * (2 * (n / 8) - 1) * 128; }
 
 // Host arithmetic of the table: the unevaluated sum of two doubles (Knuth's TwoSum, FMA product),
 // the same on every host whatever its long double is.
@@ -75,14 +86,17 @@ inline Dd64 dd64_from(long double x) {
   return {h, (double)(x - (long double)h)};
 }
 
-// The table of one axis: the header {int p}, then the blocks of K_0 .. K_6: block s
+// The table of one axis: the header {int p, growth bits, float sum |kern|}, then the blocks of K_0 .. K_6: block s
 // of a digit holds kern[(8 (s - n/8 + 1) + r - e) mod n] at row r, element e.  d: the axis' factors exp(-k_a^2 ds) at k = 0 .. n/2.
 inline void tc64_build_table(int n, const long double* d, unsigned char* dst) {
   const int h = n / 2;
   std::vector<Dd64> cs((size_t)n), r((size_t)h + 1);
-  for (int j = 0; j <= h; j++) {
-    cs[j] = dd64_from(cosl(2.0L * 3.14159265358979323846264338327950288L * j / n));
-    if (j) cs[n - j] = cs[j];
+  for (int j = 0; j <= n / 4; j++) {  // n is a multiple of 4; the other quarters by symmetry
+    const Dd64 c = dd64_from(cosl(2.0L * 3.14159265358979323846264338327950288L * j / n));
+    cs[j] = c;
+    cs[h - j] = {-c.h, -c.l};
+    cs[h + j] = {-c.h, -c.l};
+    if (j) cs[n - j] = c;
   }
   double kmax = 0.0, ksum = 0.0;
   auto mult = [&](int j) { return (j && j < n - j) ? 2 : 1; };
@@ -100,12 +114,16 @@ inline void tc64_build_table(int n, const long double* d, unsigned char* dst) {
   int p = 13;
   while (p > 0 && (kmax * ldexp(1.0, p) > 2046.0 || ksum * ldexp(1.0, p) > 8192.0 + 1e-3)) p--;
   for (int j = 0; j <= h; j++) r[j] = {ldexp(r[j].h, p), ldexp(r[j].l, p)};
-  memset(dst, 0, 16);
+  memset(dst, 0, kTc64Head);
   memcpy(dst, &p, sizeof(p));
+  const int grow = ksum < 1.999 ? 1 : 2;  // the values of a convolution stay below 2^grow of its input's largest
+  memcpy(dst + 4, &grow, sizeof(grow));
+  const float ks = (float)(ksum * 1.000001);
+  memcpy(dst + 8, &ks, sizeof(ks));
   const int nslot = 2 * (n / 8) - 1;
   std::vector<double> q((size_t)h + 1);
   std::vector<__half> q16((size_t)3 * n);  // the digit at distance j, over three periods
-  __half* out = reinterpret_cast<__half*>(dst + 16);
+  __half* out = reinterpret_cast<__half*>(dst + kTc64Head);
   for (int sl = 0; sl < 7; sl++) {
     long long sum = 0;
     for (int j = 0; j <= h; j++) {
@@ -156,20 +174,31 @@ template <int N, int KIND, int PW, int AX> constexpr size_t tc64_smem() {
          (AX == 2 ? Tc64Z<N, KIND>::BYTES : (PW == 2 ? (size_t)N * 128 * sizeof(double) : 0));
 }
 
-// The tensor-core sum t as FP64, t 2^(eb - 1085) rounded to nearest, on the integer pipe (the
-// FP64 pipe converts 2 a cycle and SM): normalised by a shift, rounded by adding the bit below
-// the last one kept (the carry runs into the exponent).  eb keeps the exponent in range.
-__device__ __forceinline__ double tc64_to_double(long long t, int eb) {
-  const unsigned long long a = (unsigned long long)(t < 0 ? -t : t);
-  const bool small = (unsigned)(a >> 32) == 0u;
-  const unsigned h = small ? (unsigned)a : (unsigned)(a >> 32), l = small ? 0u : (unsigned)a;
-  const int lz = __clz((int)h);
-  const unsigned hn = __funnelshift_l(l, h, lz), ln = l << (lz & 31);
-  const unsigned L = __funnelshift_r(ln, hn, 11);
-  const unsigned H = (hn >> 11) + ((unsigned)(eb - lz - (small ? 32 : 0)) << 20);
-  const unsigned long long r = (((unsigned long long)H << 32) | L) + ((ln >> 10) & 1u);
-  const unsigned top = (h == 0u ? 0u : (unsigned)(r >> 32)) | ((unsigned)((unsigned long long)t >> 32) & 0x80000000u);
-  return __hiloint2double((int)top, (int)(unsigned)r);
+// Tensor-core sums t as FP64, t 2^(eb - 1085) rounded to nearest, on the integer pipe (the FP64
+// pipe converts 2 a cycle and SM): normalised by a shift, rounded by adding the bit below the last
+// one kept (the carry runs into the exponent).  eb keeps the exponent in range.  A few at a time: a
+// group with a value below 2^32 (2^-30 of the scale), whose upper word is empty, takes the FP64 pipe.
+template <int K>
+__device__ __forceinline__ void tc64_to_double(const long long (&t)[K], int eb, double (&y)[K]) {
+  unsigned least = 0xffffffffu;
+#pragma unroll
+  for (int i = 0; i < K; i++) {
+    const unsigned sg = (unsigned)((int)(t[i] >> 32) >> 31);
+    // one's complement of a negative value: 1 less in the last of 62 bits
+    const unsigned h = (unsigned)(t[i] >> 32) ^ sg, l = (unsigned)t[i] ^ sg;
+    least = min(least, h);
+    const int lz = __clz((int)h);
+    const unsigned hn = __funnelshift_l(l, h, lz), ln = l << (lz & 31);
+    const unsigned L = __funnelshift_r(ln, hn, 11);
+    const unsigned H = (hn >> 11) + (unsigned)(eb - lz) * 0x100000u;
+    const unsigned long long r = (((unsigned long long)H << 32) | L) + ((ln >> 10) & 1u);
+    y[i] = __hiloint2double((int)((unsigned)(r >> 32) | (sg & 0x80000000u)), (int)(unsigned)r);
+  }
+  if (__any_sync(0xffffffffu, least == 0u)) {
+    const double sc = __hiloint2double((eb - 62) << 20, 0);
+#pragma unroll
+    for (int i = 0; i < K; i++) y[i] = (double)t[i] * sc;
+  }
 }
 // FP64 in the digits' form: X, the integer nearest x in units of 2^(eL - 1076) (eL the biased
 // exponent of the line's largest value, at least kTc64MinExp), plus the digits' biases, above 8
@@ -177,9 +206,9 @@ __device__ __forceinline__ double tc64_to_double(long long t, int eb) {
 // for the leading digit), make all digits non-negative.  Ties go to even: values of a few bits
 // below the unit meet them half of the time, and a fixed direction would shift every step's mean.
 constexpr int kTc64MinExp = 80;  // a line below 2^-943 counts as 2^-943
+constexpr unsigned long long kTc64Bias =
+    256ull * (1ull + (1ull << 9) + (1ull << 18) + (1ull << 27) + (1ull << 36)) + (512ull << 45);
 __device__ __forceinline__ unsigned long long tc64_digits(double x, int eL) {
-  constexpr unsigned long long BIAS =
-      256ull * (1ull + (1ull << 9) + (1ull << 18) + (1ull << 27) + (1ull << 36)) + (512ull << 45);
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
   const int sh = eL + 2 - (int)((hi >> 20) & 0x7ffu);  // 2 and more; a zero or subnormal: 64 and more
   const unsigned mh = __funnelshift_l(lo, (hi & 0xfffffu) | 0x100000u, 11), ml = lo << 11;  // leading bit 63
@@ -189,102 +218,163 @@ __device__ __forceinline__ unsigned long long tc64_digits(double x, int eL) {
   const unsigned wl = __funnelshift_rc(a, b, s5), wh = s5 >= 32 ? 0u : b >> s5;
   const unsigned sg = (unsigned)((int)hi >> 31);
   const unsigned long long v = (((unsigned long long)(wh ^ sg) << 32) | (wl ^ sg)) - (((unsigned long long)sg << 32) | sg);
-  return v + ((BIAS << 8) + 127ull) + (((unsigned)v >> 8) & 1u);
+  return v + ((kTc64Bias << 8) + 127ull) + (((unsigned)v >> 8) & 1u);
 }
 
-// AX 0, 1: lines along x or y; line c of the nlines starts at (c / cin) s_outer + c % cin doubles
-// and its points lie s_k apart (complex fields: real and imaginary parts are lines of their own,
-// in neighbouring threads).  AX 2: lines along z, nlines rows of N points (complex fields: two
-// rows a pencil), staged in shared memory warp by warp.
-// PW 0: the convolution; PW 1: x B_1 on q_0 = st.in, convolution; PW 2: convolution, x B_s,
-// store q_s, then (if st.Bnext) x B_{s+1}, convolution.
-template <int N, int KIND, int PW, int AX>
-__global__ void __launch_bounds__(Tc64Cfg<N>::THREADS, 1)
-kb_tc64_line(const BatchStep* __restrict__ st, int nlines, int cin, int s_outer, int s_k, int* err) {
+// Digit `dgt` (0 the leading one) of two biased integers as a pair of FP16: two bytes of each
+// that hold it, shifted and masked, as the mantissa of 1024 + digit, then exactly minus
+// (1024 + bias).
+template <int dgt> __device__ __forceinline__ uint32_t tc64_digit_pair(unsigned lo0, unsigned hi0, unsigned lo1, unsigned hi1) {
+  unsigned pk;
+  if (dgt == 5) pk = __byte_perm(lo0, lo1, 0x6521);
+  else if (dgt == 4) pk = __byte_perm(lo0, lo1, 0x7632) >> 1;
+  else if (dgt == 3) pk = __byte_perm(__funnelshift_r(lo0, hi0, 26), __funnelshift_r(lo1, hi1, 26), 0x5410);
+  else if (dgt == 2) pk = __byte_perm(hi0, hi1, 0x5410) >> 3;
+  else if (dgt == 1) pk = __byte_perm(hi0, hi1, 0x6521) >> 4;
+  else pk = __byte_perm(hi0, hi1, 0x7632) >> 5;
+  const unsigned hb = dgt == 0 ? (pk & 0x07ff07ffu) + 0x64006400u : ((pk & 0x01ff01ffu) | 0x64006400u);
+  const __half2 hv = __hsub2(*reinterpret_cast<const __half2*>(&hb),
+                             __half2half2(__ushort_as_half(dgt == 0 ? 0x6600 : 0x6500)));
+  return *reinterpret_cast<const uint32_t*>(&hv);
+}
+
+// ------------------------------------------------------------------ fixed-point fields
+// Where all three axes are on the tensor cores the field between the launches, and the
+// Boltzmann factors, are 64-bit integers (FX 1): the digits are then bit fields of the stored
+// value and the sum of the levels is the next stored value, where FP64 fields cost two
+// conversions of some twenty operations each on the integer pipe, which bounds these kernels,
+// and two FP64 multiplications a step.  One scale a launch: the field is Z 2^(E - 62), |Z| < 2^62,
+// and the launch before has left the largest |Z| (its upper word), from which this one takes the
+// shift that fills X's 54 bits.
+struct Tc64Scale {
+  int E;
+  unsigned M;  // largest upper word of |Z|
+};
+// A Boltzmann factor B in fixed point, behind this header of 256 bytes: B 2^(62 - e), complex
+// components B 2^(61 - e), e the exponent above the largest, as upper 31 bits with sign in the
+// upper word and lower 31 in the lower.
+struct Tc64Fixed {
+  int e;        // |B| < 2^e
+  int ec;       // exponent of a product with B: e + 1, complex fields e + 2
+  float m;      // the largest |B| 2^-e, rounded up (complex: of the largest real and imaginary parts)
+  int bad;      // B or the initial condition holds an infinity or a NaN
+  int wide;     // the two blocks' factors are too large for fixed point: they follow as FP64
+  int e0;       // exponent above the largest initial value (q_0 or qd_0 of the chains)
+};
+constexpr size_t kTc64FixedHeader = 256;
+constexpr int kTc64Wide = -0x7fffffff;  // Tc64Scale::E of a field in FP64
+// Between the two convolutions of a launch the scale is the field's times the factors' largest, and
+// what the values stay below it is lost from X's 54 bits: a bit or two while the largest factor is
+// below sqrt(2) (|w| ds < 0.69), but strong noise on a coarse contour (|w| ds ~ 12) lost twenty.
+
+// The largest magnitudes' upper words: mx[0], mx[1] of a's even and odd values (real and imaginary
+// parts), mx[2], mx[3] of b's, mx[4] of q's and r's (null: skipped).
+static __global__ void __launch_bounds__(256) k_tc64_max(const double2* __restrict__ a, const double2* __restrict__ b,
+                                                         const double2* __restrict__ q, const double2* __restrict__ r,
+                                                         long long n2, unsigned* __restrict__ mx) {
+  unsigned m[5] = {0u, 0u, 0u, 0u, 0u};
+  auto up = [](unsigned& o, double x) { o = max(o, (unsigned)__double2hiint(x) & 0x7fffffffu); };
+  for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n2; i += gridDim.x * 256ll) {
+    const double2 za = a[i], zb = b[i], zq = q[i];
+    up(m[0], za.x);
+    up(m[1], za.y);
+    up(m[2], zb.x);
+    up(m[3], zb.y);
+    up(m[4], zq.x);
+    up(m[4], zq.y);
+    if (r) {
+      const double2 zr = r[i];
+      up(m[4], zr.x);
+      up(m[4], zr.y);
+    }
+  }
+  __shared__ unsigned red[5];  // one global atomic a block and value, and only where it raises the value
+  if (threadIdx.x < 5) red[threadIdx.x] = 0u;
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < 5; j++) {
+    const unsigned w = __reduce_max_sync(0xffffffffu, m[j]);
+    if ((threadIdx.x & 31) == 0) atomicMax(red + j, w);
+  }
+  __syncthreads();
+  if (threadIdx.x < 5 && red[threadIdx.x] > *(volatile unsigned*)(mx + threadIdx.x))
+    atomicMax(mx + threadIdx.x, red[threadIdx.x]);
+}
+// B (both blocks) in fixed point with their headers; KIND 1: complex fields.
+template <int KIND>
+static __global__ void __launch_bounds__(256) k_tc64_fix(const double* __restrict__ a, const double* __restrict__ b,
+                                                         long long n, const unsigned* __restrict__ mx,
+                                                         char* __restrict__ fa, char* __restrict__ fb) {
+  bool bad = false;
+#pragma unroll
+  for (int j = 0; j < 5; j++) bad = bad || mx[j] >= 0x7ff00000u;
+  // sqrt(2) and more (upper word 0x3ff6a09e)
+  const bool wide = max(max(mx[0], mx[1]), max(mx[2], mx[3])) >= 0x3ff6a09eu && !bad;
+#pragma unroll
+  for (int w = 0; w < 2; w++) {
+    const double* x = w ? b : a;
+    char* f = w ? fb : fa;
+    const unsigned top = max(mx[2 * w], mx[2 * w + 1]);
+    const int e = bad ? 0 : (int)(top >> 20) - 1022;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      Tc64Fixed h;
+      h.e = e;
+      h.ec = e + 1 + KIND;
+      float m2 = 0.f;  // (the largest magnitudes 2^-e, the upper words' mantissas 2^-21 rounded up)
+#pragma unroll
+      for (int j = 0; j < 2; j++) {
+        const unsigned x = mx[2 * w + j];
+        const int down = (int)(top >> 20) - (int)(x >> 20);
+        const float f = ldexpf((float)((x & 0xfffffu) + 0x100001u) * 4.76837158203125e-7f, -down) * 1.0000002f;
+        m2 = KIND ? m2 + f * f : fmaxf(m2, f * f);
+      }
+      h.m = bad ? 1.f : sqrtf(m2) * 1.000001f;
+      h.bad = bad ? 1 : 0;
+      h.wide = wide ? 1 : 0;
+      h.e0 = bad ? 0 : (int)(mx[4] >> 20) - 1022;
+      *reinterpret_cast<Tc64Fixed*>(f) = h;
+    }
+    unsigned long long* o = reinterpret_cast<unsigned long long*>(f + kTc64FixedHeader);
+    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += gridDim.x * 256ll) {
+      const double y = bad ? 0.0 : x[i];
+      const unsigned hi = (unsigned)__double2hiint(y);
+      const int sh = (KIND ? 3 : 2) + e + 1022 - (int)((hi >> 20) & 0x7ffu);  // down from a mantissa at bit 63
+      unsigned long long mant = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | (unsigned)__double2loint(y);
+      mant = (sh > 63 || (hi & 0x7ff00000u) == 0u) ? 0ull : (mant << 11) >> sh;
+      const long long z = (hi >> 31) ? -(long long)mant : (long long)mant;
+      o[i] = wide ? (unsigned long long)__double_as_longlong(x[i])
+                  : ((unsigned long long)(unsigned)(int)(z >> 31) << 32) | ((unsigned)z & 0x7fffffffu);
+    }
+  }
+}
+
+// The tile's lines, by the warpgroups that hold them (every thread but the issuing warp's); FX 0:
+// FP64 fields and factors; FX 1: fixed point, or FP64 in its layout where `wide` says so (known
+// only after the loads of the field are on their way).
+template <int N, int KIND, int PW, int AX, int FX>
+__device__ __forceinline__ void tc64_lines(const BatchStep& s, int nlines, int cin, int s_outer, int s_k, int* err,
+                                           unsigned char* smraw, int tid, int warp, bool more, bool wide, size_t boff,
+                                           Tc64Scale in_sc, Tc64Scale* out_sc, const Tc64Fixed& hB,
+                                           const Tc64Fixed& hN) {
   using CF = Tc64Cfg<N>;
   constexpr int G = CF::G, PPT = CF::PPT, CW = CF::CW, NCH = CF::NCH, CPW = CF::CPW, NB = CF::NB, NS = CF::NS;
   constexpr uint32_t DCOL = NS * N / 2;  // first accumulator column
-  const BatchStep& s = st[blockIdx.y];
-  extern __shared__ __align__(16) unsigned char smraw[];
+  constexpr int GS = 4;                  // points converted to FP64 at a time
   int* lexp = reinterpret_cast<int*>(smraw + tc_align(CF::TAB));
   uint64_t* full = reinterpret_cast<uint64_t*>(lexp + CF::WORK);
-  uint64_t* empty = full + NCH * NB;  // full: one set a chunk, so that its readers meet every phase
+  uint64_t* empty = full + NCH * NB;
   uint64_t* done = empty + NB;
   uint32_t* tbase = reinterpret_cast<uint32_t*>(done + 1);
-  static_assert(NCH == 1 || NS % NB == 0, "a chunk's levels use every accumulator equally often");
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform
-  const bool more = PW == 2 && s.Bnext != nullptr;
-
-  // ---- table, barriers, tensor memory
-  {
-    const uint4* t4 = reinterpret_cast<const uint4*>(reinterpret_cast<const char*>(s.d[AX]) + tc_align(N * sizeof(double)));
-    uint4* d4 = reinterpret_cast<uint4*>(smraw);
-    for (int i = tid; i < CF::TAB / 16; i += CF::THREADS) d4[i] = t4[i];
-  }
-  if (tid == 0) {
-#pragma unroll
-    for (int i = 0; i < NCH * NB; i++) mbar_init(full + i, 1);
-#pragma unroll
-    for (int i = 0; i < NB; i++) mbar_init(empty + i, 4 * CPW);
-    mbar_init(done, 1);
-    mbar_init_fence();
-  }
-  if (warp == 4 * G) tc_alloc(tbase, CF::COLS);
-  fence_proxy_async_smem();
-  constexpr int NJ = NCH * NS;  // jobs a turn: (chunk, level) in order, job t in accumulator t % NB
-
-  if (warp == 4 * G) {
-    // ================================================= the issuing warp
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tm = __shfl_sync(0xffffffffu, *tbase, 0);
-    const uint64_t k0 = tc_desc(smem_addr(smraw) + 16);
-    for (int turn = 0; turn < (more ? 2 : 1); turn++) {
-      named_sync(1, CF::THREADS);  // X is in tensor memory
-      tc_fence_after();
-      for (int ch = 0; ch < NCH; ch++) {
-        for (int l = 0; l < NS; l++) {
-          const int t = ch * NS + l, b = t % NB;
-          if (t >= NB) {  // job t - NB has been read: it was use t / NB - 1 of this turn's
-            mbar_wait(empty + b, (unsigned)(turn * ((NJ - b + NB - 1) / NB) + t / NB - 1) & 1u, err, 1);
-            tc_fence_after();
-          }
-          __syncwarp();
-          if (elect_one()) {
-            const uint32_t d = tm + DCOL + (uint32_t)(b * CW);
-            const int np = l + 1 + (l == NS - 1 ? 1 : 0);
-            for (int i = 0; i < np; i++) {  // X_i K_{l-i}, and X_0 K_6 with the last level
-              const int xi = i > l ? 0 : i, kj = i > l ? NS : l - i;
-              const uint32_t a = tm + (uint32_t)(xi * (N / 2));
-              const uint64_t kd = k0 + (uint64_t)((kj * CF::NSLOT + ch * (CW / 8)) * 8);
-#pragma unroll
-              for (int j = 0; j < N / 16; j++)
-                tc_mma_f16_ts(d, a + 8 * j, kd + (N / 8 - 2 - 2 * j) * 8, tc_idesc(CW), (i > 0 || j > 0) ? 1u : 0u);
-            }
-            tc_commit(full + ch * NB + b);
-            if (t == NJ - 1) tc_commit(done);
-          }
-          __syncwarp();
-        }
-      }
-    }
-    __syncthreads();  // every accumulator has been read
-    tc_fence_after();
-    tc_dealloc(tm, CF::COLS);
-    return;
-  }
-
-  // =================================================== the lines' warpgroups
-
+  const int lane = tid & 31;
   const int g = warp >> 2, m = tid & 127;
   const int col = blockIdx.x * 128 + m;
   const bool valid = col < nlines;
   const int colc = valid ? col : 0;
-  double* F = reinterpret_cast<double*>(s.spec);
-  const double* B = reinterpret_cast<const double*>(s.B);
-  const double* Bn = reinterpret_cast<const double*>(s.Bnext);
+  double* F = reinterpret_cast<double*>(s.spec);  // FX 1: 64-bit integers, moved as doubles
+  // behind the factors' headers in the fixed-point layout
+  const double* B = reinterpret_cast<const double*>(reinterpret_cast<const char*>(s.B) + boff);
+  const double* Bn = reinterpret_cast<const double*>(reinterpret_cast<const char*>(s.Bnext) + boff);
+  const bool same = (s.Bnext == s.B);
   int base, step;
   if (AX != 2) {
     base = (colc / cin) * s_outer + (colc % cin) + g * PPT * s_k;
@@ -353,7 +443,14 @@ kb_tc64_line(const BatchStep* __restrict__ st, int nlines, int cin, int s_outer,
       zin(B);
       zwait();
 #pragma unroll
-      for (int i = 0; i < PPT; i++) v[i] = mulB(v[i], valid ? zat(i) : 0.0);
+      for (int i = 0; i < PPT; i++) {
+        double b = valid ? zat(i) : 0.0;
+        if (FX && !wide) {  // the first launch multiplies in FP64, by B 2^-e
+          const long long z = ((long long)__double2hiint(b) << 31) + (long long)__double2loint(b);
+          b = (double)z * (KIND ? 4.336808689942018e-19 : 2.168404344971009e-19);  // 2^-61, 2^-62
+        }
+        v[i] = mulB(v[i], b);
+      }
       __syncwarp();
     }
   } else {
@@ -388,64 +485,98 @@ kb_tc64_line(const BatchStep* __restrict__ st, int nlines, int cin, int s_outer,
   int ebase = 0;
   bool odd = false;
   double sc1 = 1.0, sc2 = 1.0;
-
-  auto split = [&](int turn) {
-    unsigned mx = 0;
+  // conversions back to FP64 of values below 2^(eL - 1022): results near either end of the range
+  // are scaled in two parts
+  auto set_range = [&](int eL, bool bad, int off) {
+    odd = bad || eL < 300 || eL > 1900;
+    const int eC = odd ? 1000 : eL;
+    ebase = eC + off;
+    if (odd) {
+      const int d = max(-2000, min(eL - 1000, 2000));
+      sc1 = __hiloint2double((1023 + d / 2) << 20, 0);
+      sc2 = bad ? __hiloint2double(0x7fffffff, -1) : __hiloint2double((1023 + d - d / 2) << 20, 0);
+    }
+  };
+  auto rescale = [&]() {
+#pragma unroll 1
+    for (int k = 0; k < PPT; k += 8) {
 #pragma unroll
-    for (int i = 0; i < PPT; i++) mx = max(mx, (unsigned)__double2hiint(v[i]) & 0x7fffffffu);
-    lexp[g * 128 + m] = (int)(mx >> 20);
+      for (int i = 0; i < PPT; i++)
+        if (i / 8 == k / 8) v[i] = v[i] * sc1 * sc2;
+    }
+  };
+
+  auto rest = [&](auto mode) {
+  constexpr int MODE = decltype(mode)::value;
+  const int gg = reinterpret_cast<const int*>(smraw)[1];  // growth bits of a convolution
+  // scales of the fixed-point form: the field is X 2^(eS - 54); shift: of the stored value to X's
+  // 54 bits above 8 more
+  int eS = 0, shift = 0;
+  if constexpr (MODE) {
+    if (PW == 1) {
+      eS = max(hB.e0 + KIND, kTc64MinExp - 1022);  // of q_0 B 2^-e; its digits come from FP64
+    } else {
+      shift = min(__clz((int)in_sc.M) - 2, 30);
+      eS = in_sc.E - shift;
+    }
+  }
+
+  // X into tensor memory
+  auto split = [&](int turn) {
+    int eL = 0;
+    if constexpr (!MODE) {
+      unsigned mx = 0;
+#pragma unroll
+      for (int i = 0; i < PPT; i++) mx = max(mx, (unsigned)__double2hiint(v[i]) & 0x7fffffffu);
+      lexp[g * 128 + m] = (int)(mx >> 20);
+    }
     if (turn) {  // every product of the convolution before has read X
       mbar_wait(done, 0, err, 1);
       tc_fence_after();
     }
-    named_sync(2, CF::WORK);
-    int eL = 0;
+    if constexpr (!MODE) {
+      named_sync(2, CF::WORK);
 #pragma unroll
-    for (int w = 0; w < G; w++) eL = max(eL, lexp[w * 128 + m]);
-    odd = eL < 300 || eL > 1900;
-    const bool bad = eL == 0x7ff;  // an infinity or a NaN: the line becomes NaN
-    eL = max(eL, kTc64MinExp);
-    const int eC = odd ? 1000 : eL;  // results near either end of the range: scaled in two parts
-    ebase = eC - 47 - p + 62;
-    if (odd) {
-      const int d = eL - 1000;  // -920 .. 1046
-      sc1 = __hiloint2double((1023 + d / 2) << 20, 0);
-      sc2 = bad ? __hiloint2double(0x7fffffff, -1) : __hiloint2double((1023 + d - d / 2) << 20, 0);
+      for (int w = 0; w < G; w++) eL = max(eL, lexp[w * 128 + m]);
+      const bool bad = eL == 0x7ff;  // an infinity or a NaN: the line becomes NaN
+      eL = max(eL, kTc64MinExp);
+      set_range(eL, bad, -47 - p + 62);
+    } else {
+      eL = eS + 1022;  // PW 1: the largest exponent there can be
     }
+    const unsigned mul = 1u << shift;
+    // the digits' biases, half of the 8 bits dropped, and half a unit of a product of factors (whose
+    // few bits below X's unit would meet the tie, rounded up, one time in eight)
+    const unsigned long long add = (kTc64Bias << 8) + 128ull + (turn ? (unsigned)(mul >> 1) : 0u);
 #pragma unroll
     for (int j = 0; j < PPT / 8; j++) {
       unsigned lo[8], hi[8];
 #pragma unroll
       for (int i = 0; i < 8; i++) {
-        const unsigned long long y = tc64_digits(v[8 * j + i], eL);
+        unsigned long long y;
+        if constexpr (MODE && PW != 1) {
+          const unsigned long long z = (unsigned long long)__double_as_longlong(v[8 * j + i]);
+          y = (unsigned long long)(unsigned)z * mul + add + ((unsigned long long)((unsigned)(z >> 32) * mul) << 32);
+        } else {
+          y = tc64_digits(v[8 * j + i], eL);
+        }
         lo[i] = (unsigned)y;
         hi[i] = (unsigned)(y >> 32);
       }
-#pragma unroll
-      for (int dgt = 0; dgt < NS; dgt++) {  // digit 0 is the leading one
+      auto put = [&](auto dg) {
+        constexpr int dgt = decltype(dg)::value;
         uint32_t w[4];
 #pragma unroll
-        for (int i = 0; i < 4; i++) {
-          auto dig = [&](int q) -> unsigned {
-            switch (dgt) {
-              case 5: return lo[q] >> 8;
-              case 4: return lo[q] >> 17;
-              case 3: return __funnelshift_r(lo[q], hi[q], 26);
-              case 2: return hi[q] >> 3;
-              case 1: return hi[q] >> 12;
-              default: return hi[q] >> 21;
-            }
-          };
-          const unsigned pk = __byte_perm(dig(2 * i), dig(2 * i + 1), 0x5410);
-          // FP16 1024 + digit by its bits, then exactly minus (1024 + bias)
-          const unsigned hb = dgt == 0 ? (pk & 0x07ff07ffu) + 0x64006400u : ((pk & 0x01ff01ffu) | 0x64006400u);
-          const __half2 hv = __hsub2(*reinterpret_cast<const __half2*>(&hb),
-                                     __half2half2(__ushort_as_half(dgt == 0 ? 0x6600 : 0x6500)));
-          w[i] = *reinterpret_cast<const uint32_t*>(&hv);
-        }
+        for (int i = 0; i < 4; i++) w[i] = tc64_digit_pair<dgt>(lo[2 * i], hi[2 * i], lo[2 * i + 1], hi[2 * i + 1]);
         // the two halves of each 16 points swapped
         tc_st4(tlane + (uint32_t)(dgt * (N / 2) + g * (PPT / 2) + 4 * (j ^ 1)), w);
-      }
+      };
+      put(std::integral_constant<int, 0>{});
+      put(std::integral_constant<int, 1>{});
+      put(std::integral_constant<int, 2>{});
+      put(std::integral_constant<int, 3>{});
+      put(std::integral_constant<int, 4>{});
+      put(std::integral_constant<int, 5>{});
     }
     tc_wait_st();
     tc_fence_before();
@@ -454,7 +585,11 @@ kb_tc64_line(const BatchStep* __restrict__ st, int nlines, int cin, int s_outer,
 
   const uint32_t dacc = tlane + DCOL + (uint32_t)((g % CPW) * PPT);
   long long acc[PPT];
-  // the levels of this warpgroup's chunk, added up in units of 2^-39 of level 0's
+  // the levels of this warpgroup's chunk, added up in units of 2^-39 of level 0's (level 0 first:
+  // its products are the fewest, so that the reading starts early; a 64-bit multiply-add takes
+  // the place of a sign extension and a 64-bit addition on the busier pipe)
+  int one = 1;
+  asm volatile("" : "+r"(one));
   auto collect = [&](int turn) {
 #pragma unroll
     for (int l = 0; l < NS; l++) {
@@ -468,11 +603,11 @@ kb_tc64_line(const BatchStep* __restrict__ st, int nlines, int cin, int s_outer,
         tc_wait_ld();
 #pragma unroll
         for (int i = 0; i < 8; i++) {
-          const int d = __float2int_rn(__uint_as_float(r[i]));
+          const float f = __uint_as_float(r[i]);
+          const int d = __float2int_rn(l == 5 ? f * 0.015625f : f);
           long long& a = acc[8 * j + i];
-          if (l == 0) a = (long long)((unsigned long long)(unsigned)(d << 7) << 32);
-          else if (l == 5) a += (d + 32) >> 6;
-          else a += (long long)d * (l == 1 ? (1 << 30) : (l == 2 ? (1 << 21) : (l == 3 ? (1 << 12) : (1 << 3))));
+          if (l == 0) a = (long long)((unsigned long long)(unsigned)(d * 128) << 32);
+          else a += (long long)d * (l == 1 ? (1 << 30) : (l == 2 ? (1 << 21) : (l == 3 ? (1 << 12) : (l == 4 ? (1 << 3) : one))));
         }
       }
       tc_fence_before();
@@ -481,23 +616,62 @@ kb_tc64_line(const BatchStep* __restrict__ st, int nlines, int cin, int s_outer,
         asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(empty + b)) : "memory");
     }
   };
-  // the convolution's values into v: unit 2^(eL + 1 - 1023) 2^-9 2^-p 2^-39
+  // FX 0: the convolution's values into v, unit 2^(eL + 1 - 1023) 2^-9 2^-p 2^-39
   auto finish = [&]() {
 #pragma unroll
-    for (int k = 0; k < PPT; k++) v[k] = tc64_to_double(acc[k], ebase);
-    if (odd) {
-#pragma unroll 1
-      for (int k = 0; k < PPT; k += 8) {
+    for (int j = 0; j < PPT / GS; j++) {
+      long long t[GS];
+      double y[GS];
 #pragma unroll
-        for (int i = 0; i < PPT; i++)
-          if (i / 8 == k / 8) v[i] = v[i] * sc1 * sc2;
-      }
+      for (int i = 0; i < GS; i++) t[i] = acc[GS * j + i];
+      tc64_to_double(t, ebase, y);
+#pragma unroll
+      for (int i = 0; i < GS; i++) v[GS * j + i] = y[i];
+    }
+    if (odd) rescale();
+  };
+  // FX 1: the stored form of the convolution's values, exponent eS + gg, and their largest upper word
+  auto finish_fx = [&]() {
+    const unsigned up = 1u << (14 - p - gg);
+    int mx = 0, mn = 0;
+#pragma unroll
+    for (int k = 0; k < PPT; k++) {
+      const long long z = acc[k] * up;
+      v[k] = __longlong_as_double(z);
+      mx = max(mx, (int)(z >> 32));
+      mn = min(mn, (int)(z >> 32));
+    }
+    const unsigned w = __reduce_max_sync(0xffffffffu, valid ? (unsigned)max(mx, -mn) : 0u);
+    if (lane == 0) atomicMax(lexp, (int)w);
+  };
+  // x B in fixed point, the product's unit 2^ec of x's: B as bh 2^31 + bl, x as xh 2^32 + 2 xl + 1
+  // bit, three signed 32-bit products of the four (the fourth, the bits below and the rounding down
+  // by their mean: 1 unit, for the difference of a real part 1/2).  low: half a unit less, the
+  // product's mean lies in the middle of its last unit
+  auto mulF = [&](long long x, long long b, bool low) -> long long {
+    const long long half = 1ll << 30, one_ = low ? half : 2 * half;
+    const int xh = (int)(x >> 32), xl = (int)((unsigned)x >> 1);
+    const int bh = (int)(b >> 32), bl = (int)b;
+    long long t = (long long)xl * bh + one_;
+    t += (long long)xh * bl;
+    if constexpr (KIND == 0) {
+      return (long long)xh * bh + (t >> 31);
+    } else {  // re: x b - xo bo; im: x bo + xo b
+      const int bho = __shfl_xor_sync(0xffffffffu, bh, 1), blo = __shfl_xor_sync(0xffffffffu, bl, 1);
+      const int xho = __shfl_xor_sync(0xffffffffu, xh, 1), xlo = __shfl_xor_sync(0xffffffffu, xl, 1);
+      const bool im = lane & 1;
+      // (the products of an odd lane are of x with the other's factor)
+      const int h1 = im ? bho : bh, l1 = im ? blo : bl, h2 = im ? bh : -bho, l2 = im ? bl : -blo;
+      long long u = (long long)xl * h1 + (im ? one_ : one_ - half);
+      u += (long long)xh * l1;
+      u += (long long)xlo * h2;
+      u += (long long)xho * l2;
+      return (long long)xh * h1 + ((long long)xho * h2 + (u >> 31));
     }
   };
 
   split(0);
   if constexpr (PW == 2) {
-    const bool same = (Bn == B);
     double* q = reinterpret_cast<double*>(s.out);
     if constexpr (AX == 2) {
       __syncwarp();
@@ -508,19 +682,57 @@ kb_tc64_line(const BatchStep* __restrict__ st, int nlines, int cin, int s_outer,
     }
     collect(0);
     if constexpr (AX == 2) zwait();
-    finish();
     const double* bt = area + (g * PPT) * 128 + m;
     double* qp = q + base;
+    if constexpr (MODE) {
+      set_range(eS + hB.ec + 1022, hB.bad != 0, 1);
+      const unsigned up = 1u << (14 - p);  // the convolution in units of 2^(eS - 62)
 #pragma unroll
-    for (int k = 0; k < PPT; k++) {
-      double bk;
-      if constexpr (AX == 2) bk = valid ? zat(k) : 0.0;
-      else bk = bt[k * 128];
-      const double x = mulB(v[k], bk);
-      if constexpr (AX == 2) zat(k) = x;
-      else if (valid) *qp = x;
-      qp += step;
-      v[k] = same ? mulB(x, bk) : x;
+      for (int j = 0; j < PPT / GS; j++) {  // a few points at a time: few values in flight
+        double y[GS];
+        long long x[GS], bk[GS];
+#pragma unroll
+        for (int i = 0; i < GS; i++) {
+          const int k = GS * j + i;
+          if constexpr (AX == 2) bk[i] = __double_as_longlong(valid ? zat(k) : 0.0);
+          else bk[i] = __double_as_longlong(bt[k * 128]);
+          x[i] = mulF(acc[k] * up, bk[i], false);
+        }
+        if (same) {
+#pragma unroll
+          for (int i = 0; i < GS; i++) acc[GS * j + i] = mulF(x[i], bk[i], true);
+        } else {
+#pragma unroll
+          for (int i = 0; i < GS; i++) acc[GS * j + i] = x[i];
+        }
+        tc64_to_double(x, ebase, y);
+        if (odd) {
+#pragma unroll 1
+          for (int r = 0; r < 2; r++) {
+#pragma unroll
+            for (int i = 0; i < GS; i++) y[i] *= r ? sc2 : sc1;
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < GS; i++) {
+          if constexpr (AX == 2) zat(GS * j + i) = y[i];
+          else if (valid) *qp = y[i];
+          qp += step;
+        }
+      }
+    } else {
+      finish();
+#pragma unroll
+      for (int k = 0; k < PPT; k++) {
+        double bk;
+        if constexpr (AX == 2) bk = valid ? zat(k) : 0.0;
+        else bk = bt[k * 128];
+        const double x = mulB(v[k], bk);
+        if constexpr (AX == 2) zat(k) = x;
+        else if (valid) *qp = x;
+        qp += step;
+        v[k] = same ? mulB(x, bk) : x;
+      }
     }
     if constexpr (AX == 2) zout(q);
     if (more) {
@@ -528,9 +740,20 @@ kb_tc64_line(const BatchStep* __restrict__ st, int nlines, int cin, int s_outer,
         const double* bp = Bn + base;
 #pragma unroll
         for (int k = 0; k < PPT; k++) {
-          v[k] = mulB(v[k], valid ? *bp : 0.0);
+          const double bk = valid ? *bp : 0.0;
+          if constexpr (MODE) acc[k] = mulF(acc[k], __double_as_longlong(bk), true);
+          else v[k] = mulB(v[k], bk);
           bp += step;
         }
+      }
+      if constexpr (MODE) {  // |x| <= 2^62 ks and the factors' largest, in its unit: the shift that fills X
+        // (complex: a component is at most the modulus, sqrt(2) of the components before)
+        const float bound = *(reinterpret_cast<const float*>(smraw) + 2) * hB.m * hN.m * (KIND ? 0.0884f : 0.25f);
+        const int k2 = 126 - (int)(__float_as_uint(bound) >> 23);
+        shift = max(0, min(k2, 29));
+        eS = eS + hB.ec + hN.ec - (k2 < 0 ? k2 : shift);
+#pragma unroll
+        for (int k = 0; k < PPT; k++) v[k] = __longlong_as_double(k2 < 0 ? acc[k] >> -k2 : acc[k]);
       }
       split(1);
       collect(1);
@@ -540,7 +763,8 @@ kb_tc64_line(const BatchStep* __restrict__ st, int nlines, int cin, int s_outer,
   }
   if (PW != 2 || more) {
     double* fo = F + base;
-    finish();
+    if constexpr (MODE) finish_fx();
+    else finish();
 #pragma unroll
     for (int k = 0; k < PPT; k++) {
       if constexpr (AX == 2) zat(k) = v[k];
@@ -551,6 +775,131 @@ kb_tc64_line(const BatchStep* __restrict__ st, int nlines, int cin, int s_outer,
   }
   tc_fence_before();
   __syncthreads();
+  if constexpr (MODE) {
+    if (tid == 0 && (PW != 2 || more)) {
+      atomicMax(&out_sc->M, (unsigned)*lexp);
+      if (blockIdx.x == 0) out_sc->E = eS + gg + (PW == 1 ? hB.e : 0);
+    }
+  }
+  };
+  if constexpr (FX) {
+    // (the likely form first: behind the other one its code is fetched so late that a 32^3 update
+    // takes 1.95 instead of 1.49 ms)
+    if (__builtin_expect(!wide, 1)) rest(std::integral_constant<int, 1>{});
+    else rest(std::integral_constant<int, 0>{});
+  } else {
+    rest(std::integral_constant<int, 0>{});
+  }
+}
+
+// AX 0, 1: lines along x or y; line c of the nlines starts at (c / cin) s_outer + c % cin doubles
+// and its points lie s_k apart (complex fields: real and imaginary parts are lines of their own,
+// in neighbouring threads).  AX 2: lines along z, nlines rows of N points (complex fields: two
+// rows a pencil), staged in shared memory warp by warp.
+// PW 0: the convolution; PW 1: x B_1 on q_0 = st.in, convolution; PW 2: convolution, x B_s,
+// store q_s, then (if st.Bnext) x B_{s+1}, convolution.
+// FX 0: the field and B are FP64; FX 1: the fixed-point layout, st.accA the Tc64Scale of the field
+// that the step's first launch reads, the next ones those written (PW 1 writes the first).  A march
+// whose factors are too large for it (Tc64Fixed::wide) runs FP64 fields in the same layout.
+template <int N, int KIND, int PW, int AX, int FX>
+__global__ void __launch_bounds__(Tc64Cfg<N>::THREADS, 1)
+kb_tc64_line(const BatchStep* __restrict__ st, int nlines, int cin, int s_outer, int s_k, int* err) {
+  using CF = Tc64Cfg<N>;
+  constexpr int G = CF::G, CW = CF::CW, NCH = CF::NCH, CPW = CF::CPW, NB = CF::NB, NS = CF::NS;
+  constexpr uint32_t DCOL = NS * N / 2;  // first accumulator column
+  const BatchStep& s = st[blockIdx.y];
+  extern __shared__ __align__(16) unsigned char smraw[];
+  int* lexp = reinterpret_cast<int*>(smraw + tc_align(CF::TAB));
+  uint64_t* full = reinterpret_cast<uint64_t*>(lexp + CF::WORK);
+  uint64_t* empty = full + NCH * NB;  // full: one set a chunk, so that its readers meet every phase
+  uint64_t* done = empty + NB;
+  uint32_t* tbase = reinterpret_cast<uint32_t*>(done + 1);
+  static_assert(NCH == 1 || NS % NB == 0, "a chunk's levels use every accumulator equally often");
+  const int tid = threadIdx.x;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform
+  const bool more = PW == 2 && s.Bnext != nullptr;
+
+  // ---- table, barriers, tensor memory
+  {
+    const uint4* t4 = reinterpret_cast<const uint4*>(reinterpret_cast<const char*>(s.d[AX]) + tc_align(N * sizeof(double)));
+    uint4* d4 = reinterpret_cast<uint4*>(smraw);
+    for (int i = tid; i < CF::TAB / 16; i += CF::THREADS) d4[i] = t4[i];
+  }
+  if (tid == 0) {
+    if (FX) *lexp = 0;  // largest upper word stored
+#pragma unroll
+    for (int i = 0; i < NCH * NB; i++) mbar_init(full + i, 1);
+#pragma unroll
+    for (int i = 0; i < NB; i++) mbar_init(empty + i, 4 * CPW);
+    mbar_init(done, 1);
+    mbar_init_fence();
+  }
+  if (warp == 4 * G) tc_alloc(tbase, CF::COLS);
+  fence_proxy_async_smem();
+  constexpr int NJ = NCH * NS;  // jobs a turn: (chunk, level) in order, job t in accumulator t % NB
+
+  if (warp == 4 * G) {
+    // ================================================= the issuing warp
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tm = __shfl_sync(0xffffffffu, *tbase, 0);
+    const uint64_t k0 = tc_desc(smem_addr(smraw) + kTc64Head);
+    for (int turn = 0; turn < (more ? 2 : 1); turn++) {
+      named_sync(1, CF::THREADS);  // X is in tensor memory
+      tc_fence_after();
+      for (int ch = 0; ch < NCH; ch++) {
+        for (int l = 0; l < NS; l++) {
+          const int t = ch * NS + l, b = t % NB;
+          if (t >= NB) {  // job t - NB has been read: it was use t / NB - 1 of this turn's
+            mbar_wait(empty + b, (unsigned)(turn * ((NJ - b + NB - 1) / NB) + t / NB - 1) & 1u, err, 1);
+            tc_fence_after();
+          }
+          __syncwarp();
+          if (elect_one()) {
+            const uint32_t d = tm + DCOL + (uint32_t)(b * CW);
+            const int np = l + 1 + (l == NS - 1 ? 1 : 0);
+            for (int i = 0; i < np; i++) {  // X_i K_{l-i}, and X_0 K_6 with the last level
+              const int xi = i > l ? 0 : i, kj = i > l ? NS : l - i;
+              const uint32_t a = tm + (uint32_t)(xi * (N / 2));
+              const uint64_t kd = k0 + (uint64_t)((kj * CF::NSLOT + ch * (CW / 8)) * 8);
+#pragma unroll
+              for (int j = 0; j < N / 16; j++)
+                tc_mma_f16_ts(d, a + 8 * j, kd + (N / 8 - 2 - 2 * j) * 8, tc_idesc(CW), (i > 0 || j > 0) ? 1u : 0u);
+            }
+            tc_commit(full + ch * NB + b);
+            if (t == NJ - 1) tc_commit(done);
+          }
+          __syncwarp();
+        }
+      }
+    }
+    __syncthreads();  // every accumulator has been read
+    tc_fence_after();
+    tc_dealloc(tm, CF::COLS);
+    return;
+  }
+
+  // =================================================== the lines' warpgroups
+  if constexpr (FX == 0) {
+    const Tc64Fixed none{};
+    tc64_lines<N, KIND, PW, AX, 0>(s, nlines, cin, s_outer, s_k, err, smraw, tid, warp, more, false, 0, Tc64Scale{0, 0u},
+                                   nullptr, none, none);
+  } else {
+    Tc64Scale* slot = reinterpret_cast<Tc64Scale*>(s.accA) + (PW == 2 ? 1 : 0);
+    Tc64Scale* out_sc = slot + (PW == 1 ? 0 : 1);
+    Tc64Scale in_sc{0, 0u};
+    Tc64Fixed hB{}, hN{};
+    if (PW != 1) in_sc = *slot;
+    if (PW != 0) {
+      hB = *reinterpret_cast<const Tc64Fixed*>(s.B);
+      if (more) hN = *reinterpret_cast<const Tc64Fixed*>(s.Bnext);
+    }
+    const bool wide = PW == 0 ? in_sc.E == kTc64Wide : hB.wide != 0;
+    tc64_lines<N, KIND, PW, AX, 1>(s, nlines, cin, s_outer, s_k, err, smraw, tid, warp, more, wide, kTc64FixedHeader, in_sc,
+                                   out_sc, hB, hN);
+    if (wide && tid == 0 && blockIdx.x == 0 && (PW != 2 || more)) out_sc->E = kTc64Wide;
+  }
 }
 
 }  // namespace pft

@@ -77,6 +77,15 @@ def test_matches_oracle(case):
     assert eQ <= 1e-12 and ephi <= 1e-10 and eq <= 1e-12
 
 
+@pytest.mark.parametrize("n,kind", [((32, 16, 48), SCFT), ((48, 16, 32), CL), ((16, 24, 32), SCFT)])
+def test_strong_fields(n, kind):
+    """Boltzmann factors over ten decades (fixed-point and, with the 24-point axis, FP64 factors)."""
+    wp, wm = _fields(n, kind, 730, 25.0)
+    eQ, ephi, eq = _errors(n, (4.0, 3.0, 5.0), 6, 0.5, kind, 0, wp, wm)
+    print(f"\n{n} kind={kind}: Q rel {eQ:.2e} phi abs {ephi:.2e} slices {eq:.2e}")
+    assert eQ <= 1e-12 and ephi <= 1e-10 and eq <= 1e-12
+
+
 def test_many_decades():
     """Fields that take the propagators through about twelve decades."""
     n, L, Ns, fA = (32, 48, 64), (8.0, 12.0, 16.0), 20, 0.4
