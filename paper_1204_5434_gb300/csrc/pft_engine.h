@@ -206,9 +206,9 @@ cudaError_t sepp_launch_f32(const SeppGeom& g, const BatchStep* ss, int j, int m
 cudaError_t sepp_launch_f64(const SeppGeom& g, const BatchStep* ss, int j, int members, cudaStream_t sm);
 // One convolution launch of the FP64 march on the tensor cores (pft_tc64.cuh): axis ax with the
 // Boltzmann products of its kernel (ax 0: x B_s, store, x B_{s+1}; ax 1: none; ax 2: pw 1 the
-// march's first launch, pw 2 as ax 0).  Lengths of 16, 32, 48, 64, 96 and 128 points, where it is
-// the faster of the two at every size (above that X does not fit tensor memory; other lengths are
-// no multiple of the product's 16).  The axis' table (tc64_axis_table of its factors at k = 0 ..
+// march's first launch, pw 2 as ax 0).  Lengths of 16, 32, 48, 64, 96 and 128 points (above that
+// X does not fit tensor memory; other lengths are no multiple of the product's 16); short x launches
+// stay on the FFT kernels (tc64_axis_applies).  The axis' table (tc64_axis_table of its factors at k = 0 ..
 // n/2) lies behind the factors d[ax], at the next multiple of 256 bytes.
 bool tc64_axis_applies(const SeppGeom& g, int ax);
 cudaError_t tc_launch_f64(const SeppGeom& g, const BatchStep* ss, int ax, int pw, int members, cudaStream_t sm);

@@ -58,6 +58,11 @@ CASES = [
     ((96, 64, 4), (12.0, 8.0, 0.5), 2, 0.5, CL, 1),
     ((4, 96, 64), (1.0, 12.0, 8.0), 5, 0.4, CL, 0),
     ((128, 4, 24), (8.0, 1.0, 3.0), 4, 0.6, SCFT, 0),
+    # both sides of the line below which x launches stay on the FFT kernels
+    ((64, 24, 96), (8.0, 3.0, 12.0), 2, 0.5, CL, 1),
+    ((64, 24, 64), (8.0, 3.0, 8.0), 2, 0.5, CL, 1),
+    ((16, 24, 192), (2.0, 3.0, 24.0), 2, 0.5, SCFT, 1),
+    ((16, 24, 128), (2.0, 3.0, 16.0), 2, 0.5, CL, 0),
     ((6, 128, 12), (1.5, 16.0, 3.0), 3, 0.4, CL, 1),
     ((6, 4, 128), (1.5, 1.0, 8.0), 6, 0.35, SCFT, 1),
     ((16, 192, 128), (2.0, 12.0, 8.0), 3, 0.5, SCFT, 1),
