@@ -46,11 +46,19 @@ struct BatchClass {
   pft::BatchStep* d_conc = nullptr;  // [maxNs][2K]
   pft::BatchStep* d_sep = nullptr;   // the same entries with the per-axis factors of plans 2, 3
   float tuned_ms[PFT_BATCH_PLANS] = {-1.f, -1.f, -1.f, -1.f, -1.f, -1.f, -1.f};  // autotuner timings of kBatchPlans
-  // the class's branch of the captured update: its marches, reductions and field steps
-  // run on their own stream, forked from and joined back into the batch stream, so that
-  // the classes overlap on the GPU
+};
+
+// A stream of the update besides the batch stream, with the event that joins it.
+struct BatchLane {
   cudaStream_t stream = nullptr;
-  cudaEvent_t done = nullptr;
+  cudaEvent_t event = nullptr;
+  double load = 0.0;  // work recorded on it
+};
+
+// Members k0 <= k < k1 of a class that march together.
+struct BatchGroup {
+  int cls, k0, k1;
+  double work;
 };
 
 __global__ void k_batch_increment(unsigned long long* __restrict__ c, int n) {
@@ -79,6 +87,7 @@ struct pft_batch {
   unsigned long long* d_steps = nullptr;
   int* d_err = nullptr;  // error word of the bounded waits in the separable plane kernel
   cudaEvent_t fork = nullptr;
+  std::vector<BatchLane> march, finish;
   cudaGraphExec_t graph = nullptr;
   double g_lam = -1.0, g_dt = -1.0;
   long long launches = 0;
@@ -86,6 +95,38 @@ struct pft_batch {
 };
 
 namespace {
+
+// The update's streams and the working set of a group.  A class marched whole keeps every member's
+// field, factors and newest slices in turn: 64 members of 32^3 to 64^3 are some 300 MB, so that
+// each launch found the last one's field evicted from the 129 MB L2, and the quadratures (a
+// member's own history from DRAM, a few small launches) came one after the other at the classes'
+// ends.  Groups of at most 16 MB on six streams stay in L2 together, and a member's quadrature and
+// field step run beside the other groups' marches.  Measured, ms an update with fields in and out,
+// whole classes -> groups: 16 members 6.98 -> 6.91, 32 10.4 -> 10.4, 48 22.2 -> 20.4, 64 27.3 ->
+// 25.4, 128 53.7 -> 50.8; fewer streams lose where there are few members (16 members on four
+// streams of 32 MB 8.8), larger groups gain less (64 members, six streams: 32 MB 27.6, 64 MB 28.6).
+constexpr int kMarchLanes = 6, kFinishLanes = 4;
+constexpr double kGroupBytes = 16e6;
+constexpr double kGroupSlices = 6.0;  // a member's slices: both fields, both newest slices, B_A, B_B
+
+std::vector<BatchGroup> batch_groups(const pft_batch* b) {
+  std::vector<BatchGroup> out;
+  for (size_t i = 0; i < b->classes.size(); i++) {
+    const BatchClass& c = b->classes[i];
+    const pft::CtxData& d = b->inst[c.members[0]]->d;
+    const double slice = (double)d.M * (d.prec == PFT_FP64 ? 8 : 4) * (d.kind == PFT_SCFT_REAL ? 1 : 2);
+    const int K = (int)c.members.size();
+    const int per = std::max(1, (int)(kGroupBytes / (kGroupSlices * slice)));
+    const int ng = (K + per - 1) / per;
+    for (int q = 0; q < ng; q++) {
+      BatchGroup g{(int)i, (int)((long long)K * q / ng), (int)((long long)K * (q + 1) / ng), 0.0};
+      for (int k = g.k0; k < g.k1; k++) g.work += slice * b->inst[c.members[k]]->d.Ns;
+      out.push_back(g);
+    }
+  }
+  std::stable_sort(out.begin(), out.end(), [](const BatchGroup& x, const BatchGroup& y) { return x.work > y.work; });
+  return out;
+}
 
 void batch_free(pft_batch* b) {
   if (!b) return;
@@ -95,9 +136,12 @@ void batch_free(pft_batch* b) {
     if (c.d_bwd) cudaFree(c.d_bwd);
     if (c.d_conc) cudaFree(c.d_conc);
     if (c.d_sep) cudaFree(c.d_sep);
-    if (c.stream) cudaStreamDestroy(c.stream);
-    if (c.done) cudaEventDestroy(c.done);
   }
+  for (auto* lanes : {&b->march, &b->finish})
+    for (auto& l : *lanes) {
+      if (l.stream) cudaStreamDestroy(l.stream);
+      if (l.event) cudaEventDestroy(l.event);
+    }
   if (b->fork) cudaEventDestroy(b->fork);
   if (b->d_steps) cudaFree(b->d_steps);
   if (b->d_err) cudaFree(b->d_err);
@@ -204,85 +248,123 @@ pft_status prepare_pairs(pft_batch* b, BatchClass& c) {
   return e == cudaSuccess ? PFT_OK : bcuda(e, "batch separable step table");
 }
 
-// Both marches and the densities of one class under its plan, on `sm` (the members'
-// context streams must be `sm` too).
-pft_status record_class_solve(pft_batch* b, BatchClass& c, long long* launches, cudaStream_t sm) {
+// The marches of the members k0 <= k < k1 of one class under its plan, on `sm` (the members'
+// context streams must be `sm` too); done(k) records what follows member k's marches.
+template <typename F>
+pft_status record_marches(pft_batch* b, BatchClass& c, int k0, int k1, long long* launches, cudaStream_t sm, F done) {
   const int K = (int)c.members.size();
   pft::Engine* eng = b->inst[c.members[0]]->eng;
+  const int maxNs = b->inst[c.members[k0]]->d.Ns;
+  auto active = [&](int s) { return std::min(c.active[s - 1], k1) - k0; };
+  pft_status st = PFT_OK;
   if (c.plan == 2 || (c.plan & 15) == 3) {
-    for (int j = 0; j <= c.maxNs; j++) {
-      const pft::BatchStep* st = c.d_sep + (size_t)(j == 0 ? 0 : j - 1) * 2 * K;
-      const int nact = 2 * c.active[j == 0 ? 0 : j - 1];
-      cudaError_t e = eng->batch_sep_launch(c.g, st, j, nact, c.plan, b->d_err, sm);
+    int left = k1;  // members without a recorded end: [k0, left)
+    for (int j = 0; j <= maxNs; j++) {
+      const int s = j == 0 ? 1 : j;
+      cudaError_t e = eng->batch_sep_launch(c.g, c.d_sep + ((size_t)(s - 1) * K + k0) * 2, j, 2 * active(s), c.plan,
+                                            b->d_err, sm);
       if (e != cudaSuccess) return bcuda(e, "batched separable step");
       *launches += (c.plan != 2 && j > 0) ? 2 : 1;
-    }
-    for (int i : c.members) {
-      pft_ctx* x = b->inst[i];
-      cudaError_t e = x->eng->finish_both(x->d);
-      if (e != cudaSuccess) return bcuda(e, "batched quadrature");
-      *launches += 4;
+      for (; st == PFT_OK && j > 0 && left > k0 && b->inst[c.members[left - 1]]->d.Ns == j; left--) st = done(left - 1);
+      if (st != PFT_OK) return st;
     }
     return PFT_OK;
   }
   if (c.plan == 1) {
-    for (int s = 1; s <= c.maxNs; s++) {
-      const pft::BatchStep* st = c.d_conc + (size_t)(s - 1) * 2 * K;
-      cudaError_t e = eng->batch_pair_step(c.g, st, 2 * c.active[s - 1], s == 1, sm);
+    for (int s = 1; s <= maxNs; s++) {
+      cudaError_t e = eng->batch_pair_step(c.g, c.d_conc + ((size_t)(s - 1) * K + k0) * 2, 2 * active(s), s == 1, sm);
       if (e != cudaSuccess) return bcuda(e, "batched pair step");
       *launches += eng->batch_pair_launches(c.g, s == 1);
     }
-    for (int i : c.members) {
-      pft_ctx* x = b->inst[i];
-      cudaError_t e = x->eng->solve_mid(x->d);
-      if (e == cudaSuccess) e = x->eng->quadrature(x->d);
-      if (e == cudaSuccess) e = x->eng->solve_tail(x->d);
-      if (e != cudaSuccess) return bcuda(e, "batched quadrature");
-      *launches += 6;
-    }
-    return PFT_OK;
-  }
-  for (int march = 0; march < 2; march++) {
-    for (int s = 1; s <= c.maxNs; s++) {
-      const pft::BatchStep* st = (march ? c.d_bwd : c.d_fwd) + (size_t)(s - 1) * K;
-      cudaError_t e = eng->batch_contour_step(c.g, st, c.active[s - 1], march, sm);
-      if (e != cudaSuccess) return bcuda(e, "batched contour step");
-      *launches += 5;
-    }
-    for (int i : c.members) {
-      pft_ctx* x = b->inst[i];
-      cudaError_t e = march ? x->eng->solve_tail(x->d) : x->eng->solve_mid(x->d);
-      if (e != cudaSuccess) return bcuda(e, "batched reductions");
-      *launches += march ? 2 : 3;
+  } else {
+    for (int march = 0; march < 2; march++) {
+      for (int s = 1; s <= maxNs; s++) {
+        cudaError_t e = eng->batch_contour_step(c.g, (march ? c.d_bwd : c.d_fwd) + (size_t)(s - 1) * K + k0, active(s),
+                                                march, sm);
+        if (e != cudaSuccess) return bcuda(e, "batched contour step");
+        *launches += 5;
+      }
+      for (int k = k0; k < k1 && march == 0; k++) {
+        pft_ctx* x = b->inst[c.members[k]];
+        cudaError_t e = x->eng->solve_mid(x->d);
+        if (e != cudaSuccess) return bcuda(e, "batched reductions");
+        *launches += 3;
+      }
     }
   }
-  return PFT_OK;
+  for (int k = k0; k < k1 && st == PFT_OK; k++) st = done(k);
+  return st;
 }
 
-// One field update of every instance: each class on its own stream (forked from and
-// joined back into b->stream), then the step counters on b->stream.
+// Q, the quadrature and the densities of one member after its marches, on its context's stream.
+pft_status record_finish(pft_batch* b, const BatchClass& c, int k, long long* launches) {
+  pft_ctx* x = b->inst[c.members[k]];
+  cudaError_t e = cudaSuccess;
+  if (c.plan == 0) {
+    e = x->eng->solve_tail(x->d);
+    *launches += 2;
+  } else if (c.plan == 1) {
+    e = x->eng->solve_mid(x->d);
+    if (e == cudaSuccess) e = x->eng->quadrature(x->d);
+    if (e == cudaSuccess) e = x->eng->solve_tail(x->d);
+    *launches += 6;
+  } else {
+    e = x->eng->finish_both(x->d);
+    *launches += 4;
+  }
+  return e == cudaSuccess ? PFT_OK : bcuda(e, "batched quadrature");
+}
+
+// A whole class on b->stream (the autotuner's unit).
+pft_status record_class_solve(pft_batch* b, BatchClass& c, long long* launches) {
+  return record_marches(b, c, 0, (int)c.members.size(), launches, b->stream,
+                        [&](int k) { return record_finish(b, c, k, launches); });
+}
+
+// One field update of every instance: the groups of members spread over the march streams (each
+// forked from and joined back into b->stream), each member's quadrature and field step on a finish
+// stream once its own marches are done, then the step counters on b->stream.
 pft_status record_update(pft_batch* b, double lam, double dt) {
   long long launches = 0;
   cudaError_t e = cudaEventRecord(b->fork, b->stream);
+  for (auto& l : b->march) {
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(l.stream, b->fork, 0);
+    l.load = 0.0;
+  }
+  for (auto& l : b->finish)
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(l.stream, b->fork, 0);
   if (e != cudaSuccess) return bcuda(e, "batch fork");
-  for (auto& c : b->classes) {  // plan-1 tables are prepared before any capture
-    if ((e = cudaStreamWaitEvent(c.stream, b->fork, 0)) != cudaSuccess) return bcuda(e, "class fork");
-    for (int i : c.members) b->inst[i]->d.stream = c.stream;
-    pft_status s = record_class_solve(b, c, &launches, c.stream);
-    for (int i : c.members) {
-      if (s != PFT_OK) break;
-      pft_ctx* x = b->inst[i];
+  int nf = 0;
+  for (const BatchGroup& g : batch_groups(b)) {
+    BatchClass& c = b->classes[g.cls];
+    BatchLane& l = *std::min_element(b->march.begin(), b->march.end(),
+                                     [](const BatchLane& x, const BatchLane& y) { return x.load < y.load; });
+    l.load += g.work;
+    for (int k = g.k0; k < g.k1; k++) b->inst[c.members[k]]->d.stream = l.stream;
+    pft_status s = record_marches(b, c, g.k0, g.k1, &launches, l.stream, [&](int k) {
+      pft_ctx* x = b->inst[c.members[k]];
+      BatchLane& f = b->finish[nf++ % b->finish.size()];
+      cudaError_t e = cudaEventRecord(l.event, l.stream);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(f.stream, l.event, 0);
+      if (e != cudaSuccess) return bcuda(e, "member fork");
+      x->d.stream = f.stream;
+      pft_status s = record_finish(b, c, k, &launches);
+      if (s != PFT_OK) return s;
       const bool scft = (x->d.kind == PFT_SCFT_REAL);
       e = x->eng->field_step(x->d, scft ? PFT_STEP_SCFT_EULER : PFT_STEP_CL_EULER_MARUYAMA, scft ? lam : dt, nullptr,
                              nullptr);
-      if (e != cudaSuccess) s = bcuda(e, "batched field step");
       launches += 2;
-    }
-    for (int i : c.members) b->inst[i]->d.stream = b->stream;
+      return e == cudaSuccess ? PFT_OK : bcuda(e, "batched field step");
+    });
+    for (int k = g.k0; k < g.k1; k++) b->inst[c.members[k]]->d.stream = b->stream;
     if (s != PFT_OK) return s;
-    if ((e = cudaEventRecord(c.done, c.stream)) != cudaSuccess) return bcuda(e, "class join");
-    if ((e = cudaStreamWaitEvent(b->stream, c.done, 0)) != cudaSuccess) return bcuda(e, "class join");
   }
+  for (auto* lanes : {&b->march, &b->finish})
+    for (auto& l : *lanes) {
+      if (e == cudaSuccess) e = cudaEventRecord(l.event, l.stream);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, l.event, 0);
+    }
+  if (e != cudaSuccess) return bcuda(e, "batch join");
   const int n = (int)b->inst.size();
   k_batch_increment<<<(n + 255) / 256, 256, 0, b->stream>>>(b->d_steps, n);
   launches += 1;
@@ -347,6 +429,17 @@ pft_status pft_batch_create(pft_batch** out, int count, const pft_instance_desc*
     batch_free(b);
     return bcuda(e, "batch fork event");
   }
+  b->march.resize(kMarchLanes);
+  b->finish.resize(kFinishLanes);
+  for (auto* lanes : {&b->march, &b->finish})
+    for (auto& l : *lanes) {
+      if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&l.stream, cudaStreamNonBlocking);
+      if (e == cudaSuccess) e = cudaEventCreateWithFlags(&l.event, cudaEventDisableTiming);
+    }
+  if (e != cudaSuccess) {
+    batch_free(b);
+    return bcuda(e, "batch streams");
+  }
   e = cudaMalloc(&b->d_err, 4 * sizeof(int));
   if (e == cudaSuccess) e = cudaMemsetAsync(b->d_err, 0, 4 * sizeof(int), b->stream);
   if (e != cudaSuccess) {
@@ -398,9 +491,7 @@ pft_status pft_batch_create(pft_batch** out, int count, const pft_instance_desc*
         fill_steps(b->inst[c.members[k]], s, true, &hb[(size_t)(s - 1) * K + k]);
       }
     const size_t bytes = hf.size() * sizeof(pft::BatchStep);
-    e = cudaStreamCreateWithFlags(&c.stream, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c.done, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaMalloc(&c.d_fwd, bytes);
+    e = cudaMalloc(&c.d_fwd, bytes);
     if (e == cudaSuccess) e = cudaMalloc(&c.d_bwd, bytes);
     if (e == cudaSuccess) e = cudaMemcpy(c.d_fwd, hf.data(), bytes, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(c.d_bwd, hb.data(), bytes, cudaMemcpyHostToDevice);
@@ -525,9 +616,9 @@ pft_status pft_batch_autotune(pft_batch* b) {
       c.plan = plan;
       if (plan >= 1 && (st = prepare_pairs(b, c)) != PFT_OK) break;
       long long n = 0;
-      if ((st = record_class_solve(b, c, &n, b->stream)) != PFT_OK) break;  // warm-up
+      if ((st = record_class_solve(b, c, &n)) != PFT_OK) break;  // warm-up
       cudaEventRecord(e0, b->stream);
-      if ((st = record_class_solve(b, c, &n, b->stream)) != PFT_OK) break;
+      if ((st = record_class_solve(b, c, &n)) != PFT_OK) break;
       cudaEventRecord(e1, b->stream);
       e = cudaEventSynchronize(e1);
       float ms = 0.f;

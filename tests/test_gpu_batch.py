@@ -215,3 +215,28 @@ def test_batch_plans_agree_and_autotune_picks_one(prec):
     for other in (1, 3):
         for (a0, b0), (a1, b1) in zip(out[0], out[other]):
             assert np.max(np.abs(a0 - a1)) <= tol and np.max(np.abs(b0 - b1)) <= tol
+
+
+def test_batch_groups_of_one_class():
+    """More members of one class than march together (32^3 complex FP32: ten), with equal, single-
+    step and rising contour lengths, and a second class beside it: the same as per instance, to
+    the FP32 rounding of another order of the three convolutions (a few 1e-6 after two updates)."""
+    descs = [dict(n=(32, 32, 32), L=(3.0, 3.0, 3.0), Ns=ns, fA=0.4, chiN=15.0, C=50.0, kind=CL, seed=40 + i)
+             for i, ns in enumerate((1, 5, 2, 5, 9, 3, 3, 4, 6, 7, 8, 9, 1))]
+    descs += [dict(n=(16, 16, 16), L=(3.0, 3.0, 3.0), Ns=4, fA=0.4, chiN=15.0, C=1.0, kind=SCFT, seed=60)]
+    out = []
+    for mode in (pft.PFT_BATCH_GRAPHED, pft.PFT_BATCH_PER_INSTANCE):
+        b, _ = _make(pft.PFT_FP32_MIXED, descs)
+        try:
+            pft.pft_batch_run(b, 2, LAM, DT, mode)
+            res = []
+            for i, d in enumerate(descs):
+                dt = np.float64 if d["kind"] == SCFT else np.complex128
+                gp, gm = np.empty(d["n"], dt), np.empty(d["n"], dt)
+                pft.pft_batch_get_fields(b, i, gp, gm)
+                res.append((gp, gm))
+            out.append(res)
+        finally:
+            pft.pft_batch_destroy(b)
+    for i, ((ap, am), (bp, bm)) in enumerate(zip(*out)):
+        assert np.max(np.abs(ap - bp)) <= 2e-5 and np.max(np.abs(am - bm)) <= 2e-5, i
