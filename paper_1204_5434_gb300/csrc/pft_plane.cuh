@@ -102,14 +102,14 @@ template <int N_, int E_, int R1_, int R2_> struct TwoStage<PlanX<N_, E_, R1_, R
     }
   }
   // the Stockham transform of fft() for this plan, twiddles from wr
-  template <bool INV, class X>
+  template <bool INV, int PK = 0, class X>
   __device__ static __forceinline__ void run(float2 (&v)[E], int t, const float2 (&wr)[NW], X& xch) {
 #pragma unroll
     for (int b = 0; b < NB1; b++) {
       float2 u[R1];
 #pragma unroll
       for (int r = 0; r < R1; r++) u[r] = v[b + r * NB1];
-      Dft<R1, INV, float2>::run(u);
+      Dft<R1, INV, float2>::template run<dft_pack(PK, N, 1)>(u);
       const int base = (t + b * TPC) * R1;
 #pragma unroll
       for (int r = 0; r < R1; r++) xch.put(base + r, u[r]);
@@ -128,7 +128,7 @@ template <int N_, int E_, int R1_, int R2_> struct TwoStage<PlanX<N_, E_, R1_, R
         const float2 w = wr[b * (R2 - 1) + r - 1];
         u[r] = INV ? cmulc(u[r], w) : cmul(u[r], w);
       }
-      Dft<R2, INV, float2>::run(u);
+      Dft<R2, INV, float2>::template run<dft_pack(PK, N, R1)>(u);
 #pragma unroll
       for (int r = 0; r < R2; r++) v[b + r * NB2] = u[r];
     }

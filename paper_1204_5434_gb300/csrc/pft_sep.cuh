@@ -131,10 +131,10 @@ __global__ void __launch_bounds__(SepCfg<N>::THREADS, 1) kb_sep_plane(const Batc
 
   if (MODE != 0) {
     // ---- Ky
-    fft<float, false, N>(v, ct, tws, xc);
+    fft<float, false, N, Plan<N>, 1>(v, ct, tws, xc);
 #pragma unroll
     for (int i = 0; i < E; i++) v[i] = cscale(v[i], dys[ct + TPC * i]);
-    fft<float, true, N>(v, ct, tws, xc);
+    fft<float, true, N, Plan<N>, 1>(v, ct, tws, xc);
     // transpose to the rows
 #pragma unroll
     for (int i = 0; i < E; i++) Ucol[R::ucol(ct + TPC * i, cc)] = v[i];
@@ -145,10 +145,10 @@ __global__ void __launch_bounds__(SepCfg<N>::THREADS, 1) kb_sep_plane(const Batc
       v[i] = make_float2(Ucf[R::ucol_f(L, k)], Ucf[R::ucol_f(L + H, k)]);
     }
     // ---- Kz on the row pairs
-    RT::template run<false>(v, t, wr, xr);
+    RT::template run<false, 1>(v, t, wr, xr);
 #pragma unroll
     for (int i = 0; i < E; i++) v[i] = cscale(v[i], dzs[t + TPC * i]);
-    RT::template run<true>(v, t, wr, xr);
+    RT::template run<true, 1>(v, t, wr, xr);
   } else {
     const float* q0 = reinterpret_cast<const float*>(s.in) + pbase;
 #pragma unroll
@@ -200,10 +200,10 @@ __global__ void __launch_bounds__(SepCfg<N>::THREADS, 1) kb_sep_plane(const Batc
 
   // ---- Kz of the next step
   __syncwarp();
-  RT::template run<false>(v, t, wr, xr);
+  RT::template run<false, 1>(v, t, wr, xr);
 #pragma unroll
   for (int i = 0; i < E; i++) v[i] = cscale(v[i], dzs[t + TPC * i]);
-  RT::template run<true>(v, t, wr, xr);
+  RT::template run<true, 1>(v, t, wr, xr);
   // transpose to the column pairs (each line writes only its own two rows)
 #pragma unroll
   for (int i = 0; i < E; i++) {
@@ -216,10 +216,10 @@ __global__ void __launch_bounds__(SepCfg<N>::THREADS, 1) kb_sep_plane(const Batc
   for (int i = 0; i < E; i++) v[i] = Ucol[R::ucol(ct + TPC * i, cc)];
   __syncthreads();  // every column read precedes the exchanges' writes
   // ---- Ky of the next step, then the field back to global memory
-  fft<float, false, N>(v, ct, tws, xc);
+  fft<float, false, N, Plan<N>, 1>(v, ct, tws, xc);
 #pragma unroll
   for (int i = 0; i < E; i++) v[i] = cscale(v[i], dys[ct + TPC * i]);
-  fft<float, true, N>(v, ct, tws, xc);
+  fft<float, true, N, Plan<N>, 1>(v, ct, tws, xc);
 #pragma unroll
   for (int i = 0; i < E; i++) F2[(long long)(ct + TPC * i) * H + cc] = v[i];
 }
@@ -281,10 +281,10 @@ __global__ void __launch_bounds__(SepXCfg<NX, XPL>::THREADS, SepXCfg<NX, XPL>::M
   }
   __syncthreads();  // twiddles and factors in shared memory
   XchCols<float> x{sm, C, c};
-  fft<float, false, NX, PL>(v, t, tws, x);
+  fft<float, false, NX, PL, 1>(v, t, tws, x);
 #pragma unroll
   for (int i = 0; i < E; i++) v[i] = cscale(v[i], dxs[t + TPC * i]);
-  fft<float, true, NX, PL>(v, t, tws, x);
+  fft<float, true, NX, PL, 1>(v, t, tws, x);
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();  // every thread's chunks of B_s have landed
   const bool more = (MODE == 1) && (s.Bnext != nullptr);  // no Bnext: the entry's last step
@@ -312,10 +312,10 @@ __global__ void __launch_bounds__(SepXCfg<NX, XPL>::THREADS, SepXCfg<NX, XPL>::M
     }
   }
   if (!more) return;
-  fft<float, false, NX, PL>(v, t, tws, x);
+  fft<float, false, NX, PL, 1>(v, t, tws, x);
 #pragma unroll
   for (int i = 0; i < E; i++) v[i] = cscale(v[i], dxs[t + TPC * i]);
-  fft<float, true, NX, PL>(v, t, tws, x);
+  fft<float, true, NX, PL, 1>(v, t, tws, x);
 #pragma unroll
   for (int i = 0; i < E; i++) F2[(long long)(t + TPC * i) * P + col] = v[i];
 }
@@ -413,19 +413,19 @@ __global__ void __launch_bounds__(SepCfgC<N>::THREADS, 1) kb_sep_plane_c(const B
 
   if (MODE != 0) {
     // ---- Ky on the columns, transpose, Kz on the rows
-    fft<float, false, N>(v, ct, tws, xc);
+    fft<float, false, N, Plan<N>, 1>(v, ct, tws, xc);
 #pragma unroll
     for (int i = 0; i < E; i++) v[i] = cscale(v[i], dys[ct + TPC * i]);
-    fft<float, true, N>(v, ct, tws, xc);
+    fft<float, true, N, Plan<N>, 1>(v, ct, tws, xc);
 #pragma unroll
     for (int i = 0; i < E; i++) Ucol[R::ucol(ct + TPC * i, cz)] = v[i];
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < E; i++) v[i] = Ucol[R::ucol(L, t + TPC * i)];
-    RT::template run<false>(v, t, wr, xr);
+    RT::template run<false, 1>(v, t, wr, xr);
 #pragma unroll
     for (int i = 0; i < E; i++) v[i] = cscale(v[i], dzs[t + TPC * i]);
-    RT::template run<true>(v, t, wr, xr);
+    RT::template run<true, 1>(v, t, wr, xr);
   } else {
     const float2* q0 = reinterpret_cast<const float2*>(s.in) + pbase;
 #pragma unroll
@@ -453,20 +453,20 @@ __global__ void __launch_bounds__(SepCfgC<N>::THREADS, 1) kb_sep_plane_c(const B
 
   // ---- Kz of the next step, transpose, Ky, the field back to global memory
   __syncwarp();
-  RT::template run<false>(v, t, wr, xr);
+  RT::template run<false, 1>(v, t, wr, xr);
 #pragma unroll
   for (int i = 0; i < E; i++) v[i] = cscale(v[i], dzs[t + TPC * i]);
-  RT::template run<true>(v, t, wr, xr);
+  RT::template run<true, 1>(v, t, wr, xr);
 #pragma unroll
   for (int i = 0; i < E; i++) Ucol[R::ucol(L, t + TPC * i)] = v[i];
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < E; i++) v[i] = Ucol[R::ucol(ct + TPC * i, cz)];
   __syncthreads();
-  fft<float, false, N>(v, ct, tws, xc);
+  fft<float, false, N, Plan<N>, 1>(v, ct, tws, xc);
 #pragma unroll
   for (int i = 0; i < E; i++) v[i] = cscale(v[i], dys[ct + TPC * i]);
-  fft<float, true, N>(v, ct, tws, xc);
+  fft<float, true, N, Plan<N>, 1>(v, ct, tws, xc);
 #pragma unroll
   for (int i = 0; i < E; i++) F[(long long)(ct + TPC * i) * N + cz] = v[i];
 }

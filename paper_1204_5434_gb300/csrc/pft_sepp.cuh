@@ -206,10 +206,10 @@ kb_sepp_line(const BatchStep* __restrict__ st, int nlines, int cin, int s_outer,
   };
   auto x = make_x();
   auto conv = [&]() {  // K_a: forward transform, x d_a, inverse transform
-    fft<T, false, N, PL>(v, t, tw, x);
+    fft<T, false, N, PL, 1>(v, t, tw, x);
 #pragma unroll
     for (int i = 0; i < E; i++) v[i] = cscale(v[i], d[t + TPC * i]);
-    fft<T, true, N, PL>(v, t, tw, x);
+    fft<T, true, N, PL, 1>(v, t, tw, x);
   };
   auto bsteps = [&]() -> bool {  // x B_s, store q_s, x B_{s+1}; false at the chain's end
     const Z* B = reinterpret_cast<const Z*>(s.B);
@@ -360,10 +360,10 @@ kb_sepp_z(const BatchStep* __restrict__ st, long long nlines) {
     }
   };
   auto conv = [&]() {  // Kz: forward transform, x d_z, inverse transform
-    fft<T, false, N, PL>(v, t, tw, x);
+    fft<T, false, N, PL, 1>(v, t, tw, x);
 #pragma unroll
     for (int i = 0; i < E; i++) v[i] = cscale(v[i], d[t + TPC * i]);
-    fft<T, true, N, PL>(v, t, tw, x);
+    fft<T, true, N, PL, 1>(v, t, tw, x);
   };
   auto bsteps = [&]() -> bool {  // x B_s, store q_s, x B_{s+1}; false at the chain's end
     const bool more = (s.Bnext != nullptr);
