@@ -38,8 +38,10 @@ WORK = wl.GYR128
 # conjugate step also reads the partner q and reads+writes an FP64 accumulator
 # (3e+f+2a).  Mean (5e+2f+2a)/2 with e=f=4, a=8 (FP32-mixed) or e=f=a=8 (FP64), real fields.
 BYTES_PER_UNIT = {"fp32": 22.0, "fp64": 36.0}
-# FP64 is bound by the GB300 FP64 pipe, whose rate is measured live (pft_fma_throughput,
-# a DFMA loop over every SM) as the denominator of the FP64 roofline.  Flops per unit: in the
+# FP64: the denominator is the rate of the GB300 FP64 pipe, measured live (pft_fma_throughput, a
+# DFMA loop over every SM).  The march's convolutions run on the tensor cores as exact sums of
+# integer products, so the fraction passes 1; what bounds them is the integer ALU work of splitting
+# and summing, and the tensor rate is reported beside it (22 products of 2 n flops a point and axis).  Flops per unit: in the
 # usual 5 N log2 N convention a length-n complex transform of two paired real lines costs
 # 2.5 log2(n) flops per real point, so the separable march's forward and inverse transform
 # along each of the three axes cost 5 log2(M) per point and contour step -- the same count
@@ -53,12 +55,12 @@ FP64_NOMINAL_TFLOPS = 1.25
 # previous launches left them (so each launch is charged with the write-backs its stores
 # cause).  Reads are nearly nil (the field and both factors stay in L2); the writes are the
 # q slices.  Valid only for the kernel sources it was taken on: null once any changes.
-TRAFFIC_FP32 = {"bytes_per_contour_step": 8607257.6,
+TRAFFIC_FP32 = {"bytes_per_contour_step": 8601732.3,
                 "sources": ("paper_1204_5434_gb300/csrc/pft_sep.cuh", "paper_1204_5434_gb300/csrc/pft_sepp.cuh",
                             "paper_1204_5434_gb300/csrc/pft_plane.cuh", "paper_1204_5434_gb300/csrc/pft_tma.cuh",
                             "paper_1204_5434_gb300/csrc/pft_batch.cuh", "paper_1204_5434_gb300/csrc/pft_passes.cuh",
                             "paper_1204_5434_gb300/csrc/pft_fft.cuh", "paper_1204_5434_gb300/csrc/pft_dd.cuh"),
-                "sha256": "a5c42a028a5e668d181a9e1d713064fe9e968e698dac53e4ef9fae5b65572f79"}
+                "sha256": "622725bb0755c6269af6c5cbf8c16d2728d8ebe15014ce103e9939b980a6571d"}
 
 
 def _traffic_fp32():
@@ -614,7 +616,10 @@ def run(args):
             fpu = fp64_flops_per_unit(WORK.M)
             tf = fpu * WORK.M / (step_ms * 1e-3) / 1e12
             dfma = pft.pft_fma_throughput(pft.PFT_FP64)
-            roof = {"bound": "alu", "kernel": "separable march on pencils: a y launch and an x or z launch per contour step; FP64 pipe",
+            mma = 22 * 2.0 * sum(WORK.n) * WORK.M / (step_ms * 1e-3) / 1e12
+            roof = {"bound": "alu", "kernel": "separable march on pencils: a y launch and an x or z launch per contour "
+                                              "step, convolutions on the tensor cores as exact integer products",
+                    "tensor_TFLOPs": mma,
                     "achieved": tf, "peak": dfma, "unit": "TFLOP/s", "frac": tf / dfma,
                     "peak_source": f"measured DFMA throughput of this GPU (pft_fma_throughput; nominal "
                                    f"{FP64_NOMINAL_TFLOPS} TFLOP/s)",

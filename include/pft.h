@@ -471,8 +471,8 @@ pft_status pft_launch_counts(const pft_ctx* ctx, long long* solve, long long* fi
 /* Fused multiply-add throughput of the current device, in TFLOP/s (2 flops per FMA):
  * independent FMA chains on every SM for about 20 ms, timed with CUDA events on `stream`
  * (cudaStream_t, NULL for the legacy default stream) after one warm-up launch.  No
- * counterpart in the paper: the FP64 contour step is bound by the FP64 pipe, and this is
- * the denominator of its roofline (precision PFT_FP64: DFMA; PFT_FP32_MIXED: FFMA).
+ * counterpart in the paper: the denominator of the FP64 contour step's roofline (precision
+ * PFT_FP64: DFMA; PFT_FP32_MIXED: FFMA).
  * Allocates and frees a small output buffer (stream-ordered); synchronises the stream.
  * Errors: PFT_ERR_ARG (NULL tflops, unknown precision), PFT_ERR_CUDA. */
 pft_status pft_fma_throughput(int precision, double* tflops, void* stream);

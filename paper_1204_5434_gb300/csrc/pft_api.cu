@@ -256,8 +256,8 @@ pft_status pft_create(pft_ctx** out, const pft_grid* grid, const pft_chain* chai
   d.scheme = (opts->scheme == PFT_SCHEME_RQM4) ? 1 : 0;
   d.autotune = opts->autotune != 0;
   // the default plan (measured on GB300): the separable march on the plane kernel where it
-  // applies (FP32), else the plane kernel, else the separable march on pencils (FP64: fewer
-  // passes of the FP64-pipe-bound transforms; FP32: two field round trips a contour step
+  // applies (FP32), else the plane kernel, else the separable march on pencils (FP64: the one
+  // whose convolutions run on the tensor cores; FP32: two field round trips a contour step
   // against the pencil passes' four), else the pencil passes
   if (c->eng->sep_applies(d)) d.plan_plane = 2;
   else if (c->eng->plane_applies(d)) d.plan_plane = 1;

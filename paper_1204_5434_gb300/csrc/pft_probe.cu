@@ -1,8 +1,8 @@
 // pft_probe.cu -- fused multiply-add throughput of the GPU the library runs on.
 //
-// The FP64 path of the contour step is bound by the FP64 pipe, not by HBM, so its
-// roofline denominator is the DFMA rate of the device it runs on; the FP32 rate is
-// measured the same way for comparison.  One launch of independent FMA chains over
+// The FP64 contour step is measured against the DFMA rate of the device it runs on (its
+// transforms by FFT would be bound by the FP64 pipe, not by HBM; the tensor-core march
+// passes that rate); the FP32 rate is measured the same way for comparison.  One launch of independent FMA chains over
 // every SM, timed with CUDA events after a warm-up launch.
 #include <string>
 
