@@ -868,7 +868,9 @@ kb_tc64_line(const BatchStep* __restrict__ st, int nlines, int cin, int s_outer,
                 tc_mma_f16_ts(d, a + 8 * j, kd + (N / 8 - 2 - 2 * j) * 8, tc_idesc(CW), (i > 0 || j > 0) ? 1u : 0u);
             }
             tc_commit(full + ch * NB + b);
-            if (t == NJ - 1) tc_commit(done);
+            // only where the next turn's split waits for it: an arrival that nobody waits for could
+            // come after the block has left its shared memory
+            if (t == NJ - 1 && turn == 0 && more) tc_commit(done);
           }
           __syncwarp();
         }
