@@ -25,8 +25,7 @@
  *   - PFT_FP64 runs every step to double accuracy: fields, propagators, Boltzmann factors and
  *     sums are doubles; the pencil march's convolutions along axes of 16, 32, 48, 64, 96 and
  *     128 points are exact sums of integer products on the tensor cores (values scaled by
- *     the largest of their line, or of the slice where every axis is one of these lengths;
- *     the rounding is 2^-54 of it or less).
+ *     the largest of their line, the rounding 2^-54 of it or less), rounded once to double.
  *     PFT_FP32_MIXED runs the propagators, FFTs
  *     and Boltzmann factors in float (the integrand q*qd of the contour quadrature is
  *     the float product of the two float propagators) and keeps the field update, the

@@ -104,12 +104,6 @@ struct CtxData {
   size_t ddsd_off[3] = {0, 0, 0};
   size_t ddB_off[2] = {0, 0};
   void* stepsD = nullptr;   // [2 * Ns]
-  // FP64 march on the tensor cores with fixed-point fields: the two factors, the scales of the two
-  // chains with the largest magnitudes behind them, and the step entries pointing at them
-  void* fxbuf = nullptr;
-  size_t fxB_off[2] = {0, 0};
-  size_t fxs_off = 0, fxs_bytes = 0;
-  void* stepsX = nullptr;   // [2 * Ns]
   void* stepsg = nullptr;   // [2 * Ns] BatchStep: the two spectra of the box derivative
   void* gspec = nullptr;    // [gsteps][2][Ms] spectra of a group of its steps (null: spec and spec2, one step)
   int gsteps = 1;
@@ -197,7 +191,6 @@ struct SeppGeom {
   int kind;
   int lv = 0;  // line variant: 1 = register lines (FP32, x and y lengths with a register plan)
   int* err = nullptr;  // error word of bounded waits
-  bool fx = false;     // FP64 on the tensor cores: fixed-point fields and factors
 };
 // Launch j (0..Ns) of a separable pencil march for `members` entries starting at ss (for
 // j >= 1 the entries of contour step j; j = 0 uses those of step 1).  Real fields need
@@ -214,16 +207,6 @@ bool tc64_axis_applies(const SeppGeom& g, int ax);
 cudaError_t tc_launch_f64(const SeppGeom& g, const BatchStep* ss, int ax, int pw, int members, cudaStream_t sm);
 size_t tc64_axis_table_bytes(int n);
 void tc64_axis_table(int n, const long double* d, unsigned char* dst);
-// The same with the field between the launches and the Boltzmann factors in fixed point, where
-// every axis has a table: B and Bnext of the entries point to factors made by tc64_fix (from the
-// FP64 factors a, b of n values, the initial conditions q0 and qd0 (may be null) and mx[5], zeroed; n even),
-// accA of step s to the chain's scales (zeroed before the march) at tc64_scale_step() * (s - 1).
-cudaError_t tc_launch_f64x(const SeppGeom& g, const BatchStep* ss, int ax, int pw, int members, cudaStream_t sm);
-size_t tc64_fixed_bytes(long long n);
-size_t tc64_scale_bytes(int Ns);
-size_t tc64_scale_step();
-cudaError_t tc64_fix(int kind, const double* a, const double* b, const double* q0, const double* qd0, long long n,
-                     unsigned* mx, void* fa, void* fb, int blocks, cudaStream_t sm);
 // the same march in double-float arithmetic (FP64 history, dd tables and factors)
 cudaError_t sepp_launch_dd(const SeppGeom& g, const BatchStep* ss, int j, int members, cudaStream_t sm);
 

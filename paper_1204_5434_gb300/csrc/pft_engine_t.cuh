@@ -652,64 +652,9 @@ class EngineT : public Engine {
         e = cudaMemcpy(c.stepsS, h.data(), h.size() * sizeof(BatchStep), cudaMemcpyHostToDevice);
         if (e != cudaSuccess) return e;
         if (dd_supported(c) && (e = prepare_dd(c, h)) != cudaSuccess) return e;
-        if ((e = prepare_fx(c, h)) != cudaSuccess) return e;
       }
     }
     return cudaSuccess;
-  }
-
-  // ---------------------------------------------------------------- fixed-point march
-  // The FP64 march on the tensor cores with fixed-point fields and factors (pft_tc64.cuh), where
-  // every axis has a table: the entries h of the separable march with B redirected and the scales
-  // added.  Without room for the factors (8 bytes a real value each) the FP64 fields stay.
-  cudaError_t prepare_fx(CtxData& c, std::vector<BatchStep> h) {
-    if (!std::is_same<T, double>::value || !sepp_supported(c) || c.stepsX) return cudaSuccess;
-    for (int a = 0; a < 3; a++)
-      if (!tc64_axis_table_bytes(c.n[a])) return cudaSuccess;
-    auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
-    const long long n = (c.kind == PFT_SCFT_REAL ? 1 : 2) * c.M;
-    const size_t chain = al(tc64_scale_bytes(c.Ns));
-    c.fxB_off[0] = 0;
-    c.fxB_off[1] = al(tc64_fixed_bytes(n));
-    c.fxs_off = 2 * c.fxB_off[1];
-    c.fxs_bytes = 2 * chain + 256;
-    void* buf = nullptr;
-    void* st = nullptr;
-    if (cudaMalloc(&buf, c.fxs_off + c.fxs_bytes) != cudaSuccess) {
-      (void)cudaGetLastError();
-      return cudaSuccess;
-    }
-    char* base = (char*)buf;
-    for (size_t i = 0; i < h.size(); i++) {
-      BatchStep& b = h[i];
-      const char* fB[2] = {base + c.fxB_off[0], base + c.fxB_off[1]};
-      if (b.Bnext) b.Bnext = fB[b.Bnext == c.BA ? 0 : 1];
-      if (b.B) b.B = fB[b.B == c.BA ? 0 : 1];
-      b.accA = base + c.fxs_off + (i & 1) * chain + (i / 2) * tc64_scale_step();
-    }
-    cudaError_t e = cudaMalloc(&st, h.size() * sizeof(BatchStep));
-    if (e == cudaSuccess) e = cudaMemcpy(st, h.data(), h.size() * sizeof(BatchStep), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) {
-      if (st) cudaFree(st);
-      cudaFree(buf);
-      (void)cudaGetLastError();
-      return e == cudaErrorMemoryAllocation ? cudaSuccess : e;
-    }
-    c.fxbuf = buf;
-    c.stepsX = st;
-    c.bytes += c.fxs_off + c.fxs_bytes + h.size() * sizeof(BatchStep);
-    return cudaSuccess;
-  }
-  // The factors of this solve in fixed point, the scales cleared.
-  cudaError_t start_fx(CtxData& c) {
-    char* base = (char*)c.fxbuf;
-    unsigned* mx = (unsigned*)(base + c.fxs_off + c.fxs_bytes - 256);
-    cudaError_t e = cudaMemsetAsync(base + c.fxs_off, 0, c.fxs_bytes, c.stream);
-    if (e != cudaSuccess) return e;
-    return tc64_fix(c.kind == PFT_SCFT_REAL ? 0 : 1, (const double*)c.BA, (const double*)(c.edw ? c.BA : c.BB),
-                    (const double*)c.hist, (const double*)(c.edw ? nullptr : c.qd0),
-                    (c.kind == PFT_SCFT_REAL ? 1 : 2) * c.M, mx, base + c.fxB_off[0], base + c.fxB_off[1], c.npart,
-                    c.stream);
   }
 
   // ---------------------------------------------------------------- double-float march
@@ -818,7 +763,6 @@ class EngineT : public Engine {
     g.kind = (c.kind == PFT_SCFT_REAL) ? 0 : 1;
     g.lv = (c.plan_plane == 3) ? c.plan_xv : 0;
     g.err = c.kerr;
-    g.fx = c.plan_plane == 3 && c.stepsX != nullptr;
     for (int j = 0; j <= c.Ns; j++) {
       if (members == 2) mark(c, KK_PAIR_STEP);
       const BatchStep* ss = st + (size_t)2 * (j == 0 ? 0 : j - 1);
@@ -1053,7 +997,6 @@ class EngineT : public Engine {
     const BatchStep* st = (const BatchStep*)c.steps2;
     cudaError_t e;
     if (c.plan_plane == 4 && c.stepsD && (e = split_dd(c)) != cudaSuccess) return e;
-    if (c.plan_plane == 3 && c.stepsX && (e = start_fx(c)) != cudaSuccess) return e;
     if (c.edw) {  // one reversible chain: the forward march is the whole solve
       if ((e = march_chain(c, g, st, c.stream)) != cudaSuccess) return e;
       return finish_concurrent(c);
@@ -1072,7 +1015,7 @@ class EngineT : public Engine {
       return finish_concurrent(c);
     }
     if (c.plan_plane == 3 && c.stepsS) {  // separable pencil march, both propagators per launch
-      if ((e = sepp_march(c, (const BatchStep*)(c.stepsX ? c.stepsX : c.stepsS), 2, c.stream)) != cudaSuccess) return e;
+      if ((e = sepp_march(c, (const BatchStep*)c.stepsS, 2, c.stream)) != cudaSuccess) return e;
       return finish_concurrent(c);
     }
     if (c.plan_plane == 4 && c.stepsD) {  // the same in double-float arithmetic
@@ -1125,7 +1068,7 @@ class EngineT : public Engine {
       return sep_march(c, ss, 1, sm);
     }
     if (c.plan_plane == 3 && c.stepsS) {  // separable pencil march: two launches per step
-      const BatchStep* ss = (const BatchStep*)(c.stepsX ? c.stepsX : c.stepsS) + (st - (const BatchStep*)c.steps2);
+      const BatchStep* ss = (const BatchStep*)c.stepsS + (st - (const BatchStep*)c.steps2);
       return sepp_march(c, ss, 1, sm);
     }
     if (c.plan_plane == 4 && c.stepsD) {  // the same in double-float arithmetic

@@ -494,11 +494,6 @@ cudaError_t sepp_launch_k(const SeppGeom& g, const BatchStep* ss, int j, int mem
   cudaError_t e = cudaSuccess;
   if constexpr (std::is_same<T, double>::value) {  // convolutions on the tensor cores where they apply
     const int ax = (j & 1) ? 0 : 2;
-    if (g.fx) {
-      if (j == 0) return tc_launch_f64x(g, ss, 2, 1, members, sm);
-      e = tc_launch_f64x(g, ss, 1, 0, members, sm);
-      return e != cudaSuccess ? e : tc_launch_f64x(g, ss, ax, 2, members, sm);
-    }
     if (j == 0 && tc64_axis_applies(g, 2)) return tc_launch_f64(g, ss, 2, 1, members, sm);
     if (j > 0) {
       if (tc64_axis_applies(g, 1)) {

@@ -22,15 +22,20 @@
 // read the levels before.  A line with an infinity or a NaN becomes NaN, as under the FFT.
 //
 // What bounds it: the integer pipe (64 operations a cycle and SM; ncu: busy throughout) beside the
-// products.  A 64-point tile of 128 lines takes 10,500 cycles without and 25,700 with the Boltzmann
-// products: 3,800 for the products of a convolution (2,800 at the tensor core's rate), 2,200 for the
-// digits, 7,100 for the two factors and q in FP64, 2,000 each to load and to store.  With FP64
-// fields (FX 0) 15,000 and 37,000: 4,400 for the digits, 4,200 for each conversion back, 8,200 for
-// two FP64 multiplications by B.  The FFT pair needs about 26 FP64 operations a point and
-// convolution, 13 cycles an SM, this 1.3 to 3.
-// Measured, both marches of one solve, Ns = 100, FFT pair -> FX 0 -> FX 1 (ms): 32^3 real 3.68 ->
-// 1.88 -> 1.49, 64^3 real 6.50 -> 3.29 -> 2.64, 64^3 complex 12.0 -> 4.83 -> 2.99, 128^3 real 50.5 ->
-// 13.5 -> 9.93, 128^3 complex 102.9 -> 37.2 -> 23.7.
+// products.  A 64-point tile of 128 lines takes 15,000 cycles without and 37,000 with the Boltzmann
+// products: 3,800 for the products of a convolution (2,800 at the tensor core's rate), 4,400 for the
+// digits, 4,200 for each conversion back, 8,200 for two FP64 multiplications by B, 2,000 each to
+// load and to store.  The FFT pair needs about 26 FP64 operations a point and convolution, 13
+// cycles an SM, this 1.8 to 4.  At 128 points the 17 warps' cap of 96 registers costs spills too
+// (ptxas: 648 bytes stored a thread in the fused z kernel, 628 in x, 64 in y; complex fields 316,
+// 156, 64; at most 152 at 96 points and 44 below).
+// Measured, one field update with fields in and out, FFT pair -> this (ms): 32^3 real, Ns 64, 2.49 ->
+// 1.32; 64^3 real, Ns 100, 6.59 -> 3.39, complex 12.26 -> 5.04; 128^3 real 50.9 -> 13.4, complex
+// 104.3 -> 37.0.
+// Tried: fields and factors in fixed point between the launches, one scale a slice (128^3 real 10.7
+// ms, 64^3 complex 3.3): lines and factors far below the slice's largest lose digits there, and
+// so does the block junction where the two blocks' largest factors lie apart (W- noise of 25, six
+// steps, W+ shifted by 200: 1e-9 of a slice, 1e-4 of phi); left out.
 // Tried: skipping the k steps where a digit of the kernel is zero (128 points: 26,000 -> 29,000
 // cycles, the branches cost more than a quarter of the products); the smallest level first (saves
 // two operations a point, but its eight products delay the first reading: 3,800 -> 5,100 cycles);
@@ -238,124 +243,10 @@ template <int dgt> __device__ __forceinline__ uint32_t tc64_digit_pair(unsigned 
   return *reinterpret_cast<const uint32_t*>(&hv);
 }
 
-// ------------------------------------------------------------------ fixed-point fields
-// Where all three axes are on the tensor cores the field between the launches, and the
-// Boltzmann factors, are 64-bit integers (FX 1): the digits are then bit fields of the stored
-// value and the sum of the levels is the next stored value, where FP64 fields cost two
-// conversions of some twenty operations each on the integer pipe, which bounds these kernels,
-// and two FP64 multiplications a step.  One scale a launch: the field is Z 2^(E - 62), |Z| < 2^62,
-// and the launch before has left the largest |Z| (its upper word), from which this one takes the
-// shift that fills X's 54 bits.
-struct Tc64Scale {
-  int E;
-  unsigned M;  // largest upper word of |Z|
-};
-// A Boltzmann factor B in fixed point, behind this header of 256 bytes: B 2^(62 - e), complex
-// components B 2^(61 - e), e the exponent above the largest, as upper 31 bits with sign in the
-// upper word and lower 31 in the lower.
-struct Tc64Fixed {
-  int e;        // |B| < 2^e
-  int ec;       // exponent of a product with B: e + 1, complex fields e + 2
-  float m;      // the largest |B| 2^-e, rounded up (complex: of the largest real and imaginary parts)
-  int bad;      // B or the initial condition holds an infinity or a NaN
-  int wide;     // the two blocks' factors are too large for fixed point: they follow as FP64
-  int e0;       // exponent above the largest initial value (q_0 or qd_0 of the chains)
-};
-constexpr size_t kTc64FixedHeader = 256;
-constexpr int kTc64Wide = -0x7fffffff;  // Tc64Scale::E of a field in FP64
-// Between the two convolutions of a launch the scale is the field's times the factors' largest, and
-// what the values stay below it is lost from X's 54 bits: a bit or two while the largest factor is
-// below sqrt(2) (|w| ds < 0.69), but strong noise on a coarse contour (|w| ds ~ 12) lost twenty.
-
-// The largest magnitudes' upper words: mx[0], mx[1] of a's even and odd values (real and imaginary
-// parts), mx[2], mx[3] of b's, mx[4] of q's and r's (null: skipped).
-static __global__ void __launch_bounds__(256) k_tc64_max(const double2* __restrict__ a, const double2* __restrict__ b,
-                                                         const double2* __restrict__ q, const double2* __restrict__ r,
-                                                         long long n2, unsigned* __restrict__ mx) {
-  unsigned m[5] = {0u, 0u, 0u, 0u, 0u};
-  auto up = [](unsigned& o, double x) { o = max(o, (unsigned)__double2hiint(x) & 0x7fffffffu); };
-  for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n2; i += gridDim.x * 256ll) {
-    const double2 za = a[i], zb = b[i], zq = q[i];
-    up(m[0], za.x);
-    up(m[1], za.y);
-    up(m[2], zb.x);
-    up(m[3], zb.y);
-    up(m[4], zq.x);
-    up(m[4], zq.y);
-    if (r) {
-      const double2 zr = r[i];
-      up(m[4], zr.x);
-      up(m[4], zr.y);
-    }
-  }
-  __shared__ unsigned red[5];  // one global atomic a block and value, and only where it raises the value
-  if (threadIdx.x < 5) red[threadIdx.x] = 0u;
-  __syncthreads();
-#pragma unroll
-  for (int j = 0; j < 5; j++) {
-    const unsigned w = __reduce_max_sync(0xffffffffu, m[j]);
-    if ((threadIdx.x & 31) == 0) atomicMax(red + j, w);
-  }
-  __syncthreads();
-  if (threadIdx.x < 5 && red[threadIdx.x] > *(volatile unsigned*)(mx + threadIdx.x))
-    atomicMax(mx + threadIdx.x, red[threadIdx.x]);
-}
-// B (both blocks) in fixed point with their headers; KIND 1: complex fields.
-template <int KIND>
-static __global__ void __launch_bounds__(256) k_tc64_fix(const double* __restrict__ a, const double* __restrict__ b,
-                                                         long long n, const unsigned* __restrict__ mx,
-                                                         char* __restrict__ fa, char* __restrict__ fb) {
-  bool bad = false;
-#pragma unroll
-  for (int j = 0; j < 5; j++) bad = bad || mx[j] >= 0x7ff00000u;
-  // sqrt(2) and more (upper word 0x3ff6a09e)
-  const bool wide = max(max(mx[0], mx[1]), max(mx[2], mx[3])) >= 0x3ff6a09eu && !bad;
-#pragma unroll
-  for (int w = 0; w < 2; w++) {
-    const double* x = w ? b : a;
-    char* f = w ? fb : fa;
-    const unsigned top = max(mx[2 * w], mx[2 * w + 1]);
-    const int e = bad ? 0 : (int)(top >> 20) - 1022;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-      Tc64Fixed h;
-      h.e = e;
-      h.ec = e + 1 + KIND;
-      float m2 = 0.f;  // (the largest magnitudes 2^-e, the upper words' mantissas 2^-21 rounded up)
-#pragma unroll
-      for (int j = 0; j < 2; j++) {
-        const unsigned x = mx[2 * w + j];
-        const int down = (int)(top >> 20) - (int)(x >> 20);
-        const float f = ldexpf((float)((x & 0xfffffu) + 0x100001u) * 4.76837158203125e-7f, -down) * 1.0000002f;
-        m2 = KIND ? m2 + f * f : fmaxf(m2, f * f);
-      }
-      h.m = bad ? 1.f : sqrtf(m2) * 1.000001f;
-      h.bad = bad ? 1 : 0;
-      h.wide = wide ? 1 : 0;
-      h.e0 = bad ? 0 : (int)(mx[4] >> 20) - 1022;
-      *reinterpret_cast<Tc64Fixed*>(f) = h;
-    }
-    unsigned long long* o = reinterpret_cast<unsigned long long*>(f + kTc64FixedHeader);
-    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += gridDim.x * 256ll) {
-      const double y = bad ? 0.0 : x[i];
-      const unsigned hi = (unsigned)__double2hiint(y);
-      const int sh = (KIND ? 3 : 2) + e + 1022 - (int)((hi >> 20) & 0x7ffu);  // down from a mantissa at bit 63
-      unsigned long long mant = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | (unsigned)__double2loint(y);
-      mant = (sh > 63 || (hi & 0x7ff00000u) == 0u) ? 0ull : (mant << 11) >> sh;
-      const long long z = (hi >> 31) ? -(long long)mant : (long long)mant;
-      o[i] = wide ? (unsigned long long)__double_as_longlong(x[i])
-                  : ((unsigned long long)(unsigned)(int)(z >> 31) << 32) | ((unsigned)z & 0x7fffffffu);
-    }
-  }
-}
-
-// The tile's lines, by the warpgroups that hold them (every thread but the issuing warp's); FX 0:
-// FP64 fields and factors; FX 1: fixed point, or FP64 in its layout where `wide` says so (known
-// only after the loads of the field are on their way).
-template <int N, int KIND, int PW, int AX, int FX>
+// The tile's lines, by the warpgroups that hold them (every thread but the issuing warp's).
+template <int N, int KIND, int PW, int AX>
 __device__ __forceinline__ void tc64_lines(const BatchStep& s, int nlines, int cin, int s_outer, int s_k, int* err,
-                                           unsigned char* smraw, int tid, int warp, bool more, bool wide, size_t boff,
-                                           Tc64Scale in_sc, Tc64Scale* out_sc, const Tc64Fixed& hB,
-                                           const Tc64Fixed& hN) {
+                                           unsigned char* smraw, int tid, int warp, bool more) {
   using CF = Tc64Cfg<N>;
   constexpr int G = CF::G, PPT = CF::PPT, CW = CF::CW, NCH = CF::NCH, CPW = CF::CPW, NB = CF::NB, NS = CF::NS;
   constexpr uint32_t DCOL = NS * N / 2;  // first accumulator column
@@ -370,10 +261,9 @@ __device__ __forceinline__ void tc64_lines(const BatchStep& s, int nlines, int c
   const int col = blockIdx.x * 128 + m;
   const bool valid = col < nlines;
   const int colc = valid ? col : 0;
-  double* F = reinterpret_cast<double*>(s.spec);  // FX 1: 64-bit integers, moved as doubles
-  // behind the factors' headers in the fixed-point layout
-  const double* B = reinterpret_cast<const double*>(reinterpret_cast<const char*>(s.B) + boff);
-  const double* Bn = reinterpret_cast<const double*>(reinterpret_cast<const char*>(s.Bnext) + boff);
+  double* F = reinterpret_cast<double*>(s.spec);
+  const double* B = reinterpret_cast<const double*>(s.B);
+  const double* Bn = reinterpret_cast<const double*>(s.Bnext);
   const bool same = (s.Bnext == s.B);
   int base, step;
   if (AX != 2) {
@@ -443,14 +333,7 @@ __device__ __forceinline__ void tc64_lines(const BatchStep& s, int nlines, int c
       zin(B);
       zwait();
 #pragma unroll
-      for (int i = 0; i < PPT; i++) {
-        double b = valid ? zat(i) : 0.0;
-        if (FX && !wide) {  // the first launch multiplies in FP64, by B 2^-e
-          const long long z = ((long long)__double2hiint(b) << 31) + (long long)__double2loint(b);
-          b = (double)z * (KIND ? 4.336808689942018e-19 : 2.168404344971009e-19);  // 2^-61, 2^-62
-        }
-        v[i] = mulB(v[i], b);
-      }
+      for (int i = 0; i < PPT; i++) v[i] = mulB(v[i], valid ? zat(i) : 0.0);
       __syncwarp();
     }
   } else {
@@ -487,79 +370,40 @@ __device__ __forceinline__ void tc64_lines(const BatchStep& s, int nlines, int c
   double sc1 = 1.0, sc2 = 1.0;
   // conversions back to FP64 of values below 2^(eL - 1022): results near either end of the range
   // are scaled in two parts
-  auto set_range = [&](int eL, bool bad, int off) {
+  auto set_range = [&](int eL, bool bad) {
     odd = bad || eL < 300 || eL > 1900;
     const int eC = odd ? 1000 : eL;
-    ebase = eC + off;
+    ebase = eC - 47 - p + 62;
     if (odd) {
       const int d = max(-2000, min(eL - 1000, 2000));
       sc1 = __hiloint2double((1023 + d / 2) << 20, 0);
       sc2 = bad ? __hiloint2double(0x7fffffff, -1) : __hiloint2double((1023 + d - d / 2) << 20, 0);
     }
   };
-  auto rescale = [&]() {
-#pragma unroll 1
-    for (int k = 0; k < PPT; k += 8) {
-#pragma unroll
-      for (int i = 0; i < PPT; i++)
-        if (i / 8 == k / 8) v[i] = v[i] * sc1 * sc2;
-    }
-  };
-
-  auto rest = [&](auto mode) {
-  constexpr int MODE = decltype(mode)::value;
-  const int gg = reinterpret_cast<const int*>(smraw)[1];  // growth bits of a convolution
-  // scales of the fixed-point form: the field is X 2^(eS - 54); shift: of the stored value to X's
-  // 54 bits above 8 more
-  int eS = 0, shift = 0;
-  if constexpr (MODE) {
-    if (PW == 1) {
-      eS = max(hB.e0 + KIND, kTc64MinExp - 1022);  // of q_0 B 2^-e; its digits come from FP64
-    } else {
-      shift = min(__clz((int)in_sc.M) - 2, 30);
-      eS = in_sc.E - shift;
-    }
-  }
 
   // X into tensor memory
   auto split = [&](int turn) {
-    int eL = 0;
-    if constexpr (!MODE) {
-      unsigned mx = 0;
+    unsigned mx = 0;
 #pragma unroll
-      for (int i = 0; i < PPT; i++) mx = max(mx, (unsigned)__double2hiint(v[i]) & 0x7fffffffu);
-      lexp[g * 128 + m] = (int)(mx >> 20);
-    }
+    for (int i = 0; i < PPT; i++) mx = max(mx, (unsigned)__double2hiint(v[i]) & 0x7fffffffu);
+    lexp[g * 128 + m] = (int)(mx >> 20);
     if (turn) {  // every product of the convolution before has read X
       mbar_wait(done, 0, err, 1);
       tc_fence_after();
     }
-    if constexpr (!MODE) {
-      named_sync(2, CF::WORK);
+    named_sync(2, CF::WORK);
+    int eL = 0;
 #pragma unroll
-      for (int w = 0; w < G; w++) eL = max(eL, lexp[w * 128 + m]);
-      const bool bad = eL == 0x7ff;  // an infinity or a NaN: the line becomes NaN
-      eL = max(eL, kTc64MinExp);
-      set_range(eL, bad, -47 - p + 62);
-    } else {
-      eL = eS + 1022;  // PW 1: the largest exponent there can be
-    }
-    const unsigned mul = 1u << shift;
-    // the digits' biases, half of the 8 bits dropped, and half a unit of a product of factors (whose
-    // few bits below X's unit would meet the tie, rounded up, one time in eight)
-    const unsigned long long add = (kTc64Bias << 8) + 128ull + (turn ? (unsigned)(mul >> 1) : 0u);
+    for (int w = 0; w < G; w++) eL = max(eL, lexp[w * 128 + m]);
+    const bool bad = eL == 0x7ff;  // an infinity or a NaN: the line becomes NaN
+    eL = max(eL, kTc64MinExp);
+    set_range(eL, bad);
 #pragma unroll
     for (int j = 0; j < PPT / 8; j++) {
       unsigned lo[8], hi[8];
 #pragma unroll
       for (int i = 0; i < 8; i++) {
-        unsigned long long y;
-        if constexpr (MODE && PW != 1) {
-          const unsigned long long z = (unsigned long long)__double_as_longlong(v[8 * j + i]);
-          y = (unsigned long long)(unsigned)z * mul + add + ((unsigned long long)((unsigned)(z >> 32) * mul) << 32);
-        } else {
-          y = tc64_digits(v[8 * j + i], eL);
-        }
+        const unsigned long long y = tc64_digits(v[8 * j + i], eL);
         lo[i] = (unsigned)y;
         hi[i] = (unsigned)(y >> 32);
       }
@@ -616,7 +460,7 @@ __device__ __forceinline__ void tc64_lines(const BatchStep& s, int nlines, int c
         asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(empty + b)) : "memory");
     }
   };
-  // FX 0: the convolution's values into v, unit 2^(eL + 1 - 1023) 2^-9 2^-p 2^-39
+  // the convolution's values into v, unit 2^(eL + 1 - 1023) 2^-9 2^-p 2^-39
   auto finish = [&]() {
 #pragma unroll
     for (int j = 0; j < PPT / GS; j++) {
@@ -628,45 +472,13 @@ __device__ __forceinline__ void tc64_lines(const BatchStep& s, int nlines, int c
 #pragma unroll
       for (int i = 0; i < GS; i++) v[GS * j + i] = y[i];
     }
-    if (odd) rescale();
-  };
-  // FX 1: the stored form of the convolution's values, exponent eS + gg, and their largest upper word
-  auto finish_fx = [&]() {
-    const unsigned up = 1u << (14 - p - gg);
-    int mx = 0, mn = 0;
+    if (odd) {
+#pragma unroll 1
+      for (int k = 0; k < PPT; k += 8) {
 #pragma unroll
-    for (int k = 0; k < PPT; k++) {
-      const long long z = acc[k] * up;
-      v[k] = __longlong_as_double(z);
-      mx = max(mx, (int)(z >> 32));
-      mn = min(mn, (int)(z >> 32));
-    }
-    const unsigned w = __reduce_max_sync(0xffffffffu, valid ? (unsigned)max(mx, -mn) : 0u);
-    if (lane == 0) atomicMax(lexp, (int)w);
-  };
-  // x B in fixed point, the product's unit 2^ec of x's: B as bh 2^31 + bl, x as xh 2^32 + 2 xl + 1
-  // bit, three signed 32-bit products of the four (the fourth, the bits below and the rounding down
-  // by their mean: 1 unit, for the difference of a real part 1/2).  low: half a unit less, the
-  // product's mean lies in the middle of its last unit
-  auto mulF = [&](long long x, long long b, bool low) -> long long {
-    const long long half = 1ll << 30, one_ = low ? half : 2 * half;
-    const int xh = (int)(x >> 32), xl = (int)((unsigned)x >> 1);
-    const int bh = (int)(b >> 32), bl = (int)b;
-    long long t = (long long)xl * bh + one_;
-    t += (long long)xh * bl;
-    if constexpr (KIND == 0) {
-      return (long long)xh * bh + (t >> 31);
-    } else {  // re: x b - xo bo; im: x bo + xo b
-      const int bho = __shfl_xor_sync(0xffffffffu, bh, 1), blo = __shfl_xor_sync(0xffffffffu, bl, 1);
-      const int xho = __shfl_xor_sync(0xffffffffu, xh, 1), xlo = __shfl_xor_sync(0xffffffffu, xl, 1);
-      const bool im = lane & 1;
-      // (the products of an odd lane are of x with the other's factor)
-      const int h1 = im ? bho : bh, l1 = im ? blo : bl, h2 = im ? bh : -bho, l2 = im ? bl : -blo;
-      long long u = (long long)xl * h1 + (im ? one_ : one_ - half);
-      u += (long long)xh * l1;
-      u += (long long)xlo * h2;
-      u += (long long)xho * l2;
-      return (long long)xh * h1 + ((long long)xho * h2 + (u >> 31));
+        for (int i = 0; i < PPT; i++)
+          if (i / 8 == k / 8) v[i] = v[i] * sc1 * sc2;
+      }
     }
   };
 
@@ -684,55 +496,17 @@ __device__ __forceinline__ void tc64_lines(const BatchStep& s, int nlines, int c
     if constexpr (AX == 2) zwait();
     const double* bt = area + (g * PPT) * 128 + m;
     double* qp = q + base;
-    if constexpr (MODE) {
-      set_range(eS + hB.ec + 1022, hB.bad != 0, 1);
-      const unsigned up = 1u << (14 - p);  // the convolution in units of 2^(eS - 62)
+    finish();
 #pragma unroll
-      for (int j = 0; j < PPT / GS; j++) {  // a few points at a time: few values in flight
-        double y[GS];
-        long long x[GS], bk[GS];
-#pragma unroll
-        for (int i = 0; i < GS; i++) {
-          const int k = GS * j + i;
-          if constexpr (AX == 2) bk[i] = __double_as_longlong(valid ? zat(k) : 0.0);
-          else bk[i] = __double_as_longlong(bt[k * 128]);
-          x[i] = mulF(acc[k] * up, bk[i], false);
-        }
-        if (same) {
-#pragma unroll
-          for (int i = 0; i < GS; i++) acc[GS * j + i] = mulF(x[i], bk[i], true);
-        } else {
-#pragma unroll
-          for (int i = 0; i < GS; i++) acc[GS * j + i] = x[i];
-        }
-        tc64_to_double(x, ebase, y);
-        if (odd) {
-#pragma unroll 1
-          for (int r = 0; r < 2; r++) {
-#pragma unroll
-            for (int i = 0; i < GS; i++) y[i] *= r ? sc2 : sc1;
-          }
-        }
-#pragma unroll
-        for (int i = 0; i < GS; i++) {
-          if constexpr (AX == 2) zat(GS * j + i) = y[i];
-          else if (valid) *qp = y[i];
-          qp += step;
-        }
-      }
-    } else {
-      finish();
-#pragma unroll
-      for (int k = 0; k < PPT; k++) {
-        double bk;
-        if constexpr (AX == 2) bk = valid ? zat(k) : 0.0;
-        else bk = bt[k * 128];
-        const double x = mulB(v[k], bk);
-        if constexpr (AX == 2) zat(k) = x;
-        else if (valid) *qp = x;
-        qp += step;
-        v[k] = same ? mulB(x, bk) : x;
-      }
+    for (int k = 0; k < PPT; k++) {
+      double bk;
+      if constexpr (AX == 2) bk = valid ? zat(k) : 0.0;
+      else bk = bt[k * 128];
+      const double x = mulB(v[k], bk);
+      if constexpr (AX == 2) zat(k) = x;
+      else if (valid) *qp = x;
+      qp += step;
+      v[k] = same ? mulB(x, bk) : x;
     }
     if constexpr (AX == 2) zout(q);
     if (more) {
@@ -740,20 +514,9 @@ __device__ __forceinline__ void tc64_lines(const BatchStep& s, int nlines, int c
         const double* bp = Bn + base;
 #pragma unroll
         for (int k = 0; k < PPT; k++) {
-          const double bk = valid ? *bp : 0.0;
-          if constexpr (MODE) acc[k] = mulF(acc[k], __double_as_longlong(bk), true);
-          else v[k] = mulB(v[k], bk);
+          v[k] = mulB(v[k], valid ? *bp : 0.0);
           bp += step;
         }
-      }
-      if constexpr (MODE) {  // |x| <= 2^62 ks and the factors' largest, in its unit: the shift that fills X
-        // (complex: a component is at most the modulus, sqrt(2) of the components before)
-        const float bound = *(reinterpret_cast<const float*>(smraw) + 2) * hB.m * hN.m * (KIND ? 0.0884f : 0.25f);
-        const int k2 = 126 - (int)(__float_as_uint(bound) >> 23);
-        shift = max(0, min(k2, 29));
-        eS = eS + hB.ec + hN.ec - (k2 < 0 ? k2 : shift);
-#pragma unroll
-        for (int k = 0; k < PPT; k++) v[k] = __longlong_as_double(k2 < 0 ? acc[k] >> -k2 : acc[k]);
       }
       split(1);
       collect(1);
@@ -763,8 +526,7 @@ __device__ __forceinline__ void tc64_lines(const BatchStep& s, int nlines, int c
   }
   if (PW != 2 || more) {
     double* fo = F + base;
-    if constexpr (MODE) finish_fx();
-    else finish();
+    finish();
 #pragma unroll
     for (int k = 0; k < PPT; k++) {
       if constexpr (AX == 2) zat(k) = v[k];
@@ -775,21 +537,6 @@ __device__ __forceinline__ void tc64_lines(const BatchStep& s, int nlines, int c
   }
   tc_fence_before();
   __syncthreads();
-  if constexpr (MODE) {
-    if (tid == 0 && (PW != 2 || more)) {
-      atomicMax(&out_sc->M, (unsigned)*lexp);
-      if (blockIdx.x == 0) out_sc->E = eS + gg + (PW == 1 ? hB.e : 0);
-    }
-  }
-  };
-  if constexpr (FX) {
-    // (the likely form first: behind the other one its code is fetched so late that a 32^3 update
-    // takes 1.95 instead of 1.49 ms)
-    if (__builtin_expect(!wide, 1)) rest(std::integral_constant<int, 1>{});
-    else rest(std::integral_constant<int, 0>{});
-  } else {
-    rest(std::integral_constant<int, 0>{});
-  }
 }
 
 // AX 0, 1: lines along x or y; line c of the nlines starts at (c / cin) s_outer + c % cin doubles
@@ -798,10 +545,7 @@ __device__ __forceinline__ void tc64_lines(const BatchStep& s, int nlines, int c
 // rows a pencil), staged in shared memory warp by warp.
 // PW 0: the convolution; PW 1: x B_1 on q_0 = st.in, convolution; PW 2: convolution, x B_s,
 // store q_s, then (if st.Bnext) x B_{s+1}, convolution.
-// FX 0: the field and B are FP64; FX 1: the fixed-point layout, st.accA the Tc64Scale of the field
-// that the step's first launch reads, the next ones those written (PW 1 writes the first).  A march
-// whose factors are too large for it (Tc64Fixed::wide) runs FP64 fields in the same layout.
-template <int N, int KIND, int PW, int AX, int FX>
+template <int N, int KIND, int PW, int AX>
 __global__ void __launch_bounds__(Tc64Cfg<N>::THREADS, 1)
 kb_tc64_line(const BatchStep* __restrict__ st, int nlines, int cin, int s_outer, int s_k, int* err) {
   using CF = Tc64Cfg<N>;
@@ -826,7 +570,6 @@ kb_tc64_line(const BatchStep* __restrict__ st, int nlines, int cin, int s_outer,
     for (int i = tid; i < CF::TAB / 16; i += CF::THREADS) d4[i] = t4[i];
   }
   if (tid == 0) {
-    if (FX) *lexp = 0;  // largest upper word stored
 #pragma unroll
     for (int i = 0; i < NCH * NB; i++) mbar_init(full + i, 1);
 #pragma unroll
@@ -883,25 +626,7 @@ kb_tc64_line(const BatchStep* __restrict__ st, int nlines, int cin, int s_outer,
   }
 
   // =================================================== the lines' warpgroups
-  if constexpr (FX == 0) {
-    const Tc64Fixed none{};
-    tc64_lines<N, KIND, PW, AX, 0>(s, nlines, cin, s_outer, s_k, err, smraw, tid, warp, more, false, 0, Tc64Scale{0, 0u},
-                                   nullptr, none, none);
-  } else {
-    Tc64Scale* slot = reinterpret_cast<Tc64Scale*>(s.accA) + (PW == 2 ? 1 : 0);
-    Tc64Scale* out_sc = slot + (PW == 1 ? 0 : 1);
-    Tc64Scale in_sc{0, 0u};
-    Tc64Fixed hB{}, hN{};
-    if (PW != 1) in_sc = *slot;
-    if (PW != 0) {
-      hB = *reinterpret_cast<const Tc64Fixed*>(s.B);
-      if (more) hN = *reinterpret_cast<const Tc64Fixed*>(s.Bnext);
-    }
-    const bool wide = PW == 0 ? in_sc.E == kTc64Wide : hB.wide != 0;
-    tc64_lines<N, KIND, PW, AX, 1>(s, nlines, cin, s_outer, s_k, err, smraw, tid, warp, more, wide, kTc64FixedHeader, in_sc,
-                                   out_sc, hB, hN);
-    if (wide && tid == 0 && blockIdx.x == 0 && (PW != 2 || more)) out_sc->E = kTc64Wide;
-  }
+  tc64_lines<N, KIND, PW, AX>(s, nlines, cin, s_outer, s_k, err, smraw, tid, warp, more);
 }
 
 }  // namespace pft

@@ -22,7 +22,7 @@ bool tc64_axis_applies(const SeppGeom& g, int ax) {
   return g.kind == 0 || g.n[0] < 64 || lines >= 2048;
 }
 cudaError_t tc_launch_f64(const SeppGeom& g, const BatchStep* ss, int ax, int pw, int members, cudaStream_t sm) {
-  return g.kind == 0 ? tc64_axis_k<0, 0>(g, ss, ax, pw, members, sm) : tc_launch_f64c(g, ss, ax, pw, members, sm);
+  return g.kind == 0 ? tc64_axis_k<0>(g, ss, ax, pw, members, sm) : tc_launch_f64c(g, ss, ax, pw, members, sm);
 }
 size_t tc64_axis_table_bytes(int n) { return tc64_axis_ok(n) ? tc64_table_bytes(n) : 0; }
 void tc64_axis_table(int n, const long double* d, unsigned char* dst) { tc64_build_table(n, d, dst); }
