@@ -179,8 +179,10 @@ class EngineT : public Engine {
         const double k = 2.0 * M_PI * (double)mm / c.L[a];
         sd[m] = (T)(exp(-k * k * c.ds) / (double)na);
       }
-      // the axis' table of the tensor-core convolution; an axis like an earlier one shares its values
-      const size_t tcb = std::is_same<T, double>::value ? tc64_axis_table_bytes(na) : 0;
+      // the axis' table of the tensor-core convolution, where a march may use it; an axis like an
+      // earlier one shares its values
+      const bool tcu = std::is_same<T, double>::value && c.scheme == 0 && sepp_supported(c);
+      const size_t tcb = tcu ? tc64_axis_table_bytes(na) : 0;
       unsigned char* tct = h.data() + c.sd_off[a] + al(sizeof(T) * (size_t)na);
       int like = -1;
       for (int b = 0; b < a; b++)

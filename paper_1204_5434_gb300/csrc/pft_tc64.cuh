@@ -91,11 +91,10 @@ inline Dd64 dd64_from(long double x) {
   return {h, (double)(x - (long double)h)};
 }
 
-// The table of one axis: the header {int p, growth bits, float sum |kern|}, then the blocks of K_0 .. K_6: block s
-// of a digit holds kern[(8 (s - n/8 + 1) + r - e) mod n] at row r, element e.  d: the axis' factors exp(-k_a^2 ds) at k = 0 .. n/2.
-inline void tc64_build_table(int n, const long double* d, unsigned char* dst) {
+// cos(2 pi j / n), j = 0 .. n-1, made once a length: long double is software on aarch64.
+inline std::vector<Dd64> tc64_make_cosines(int n) {
   const int h = n / 2;
-  std::vector<Dd64> cs((size_t)n), r((size_t)h + 1);
+  std::vector<Dd64> cs((size_t)n);
   for (int j = 0; j <= n / 4; j++) {  // n is a multiple of 4; the other quarters by symmetry
     const Dd64 c = dd64_from(cosl(2.0L * 3.14159265358979323846264338327950288L * j / n));
     cs[j] = c;
@@ -103,17 +102,41 @@ inline void tc64_build_table(int n, const long double* d, unsigned char* dst) {
     cs[h + j] = {-c.h, -c.l};
     if (j) cs[n - j] = c;
   }
-  double kmax = 0.0, ksum = 0.0;
+  return cs;
+}
+inline const std::vector<Dd64>& tc64_cosines(int n) {
+  static const std::vector<Dd64> c16 = tc64_make_cosines(16), c32 = tc64_make_cosines(32), c48 = tc64_make_cosines(48),
+                                 c64 = tc64_make_cosines(64), c96 = tc64_make_cosines(96), c128 = tc64_make_cosines(128);
+  switch (n) {
+    case 16: return c16;
+    case 32: return c32;
+    case 48: return c48;
+    case 64: return c64;
+    case 96: return c96;
+    default: return c128;
+  }
+}
+
+// The table of one axis: the header {int p, growth bits, float sum |kern|}, then the blocks of K_0 .. K_6: block s
+// of a digit holds kern[(8 (s - n/8 + 1) + r - e) mod n] at row r, element e.  d: the axis' factors exp(-k_a^2 ds) at k = 0 .. n/2.
+inline void tc64_build_table(int n, const long double* d, unsigned char* dst) {
+  const int h = n / 2;
+  const std::vector<Dd64>& cs = tc64_cosines(n);
   auto mult = [&](int j) { return (j && j < n - j) ? 2 : 1; };
-  for (int j = 0; j <= h; j++) {
-    Dd64 a = {0.0, 0.0};
-    for (int k = 0; k <= h; k++) {
-      const Dd64 f = dd64_from(d[k] * (mult(k) / (long double)n));
-      a = dd64_add(a, dd64_mul(f, cs[(size_t)((j * k) % n)]));
+  // (k outside: the sums of the j are independent of one another, a chain of additions each)
+  std::vector<Dd64> r((size_t)h + 1, Dd64{0.0, 0.0});
+  for (int k = 0; k <= h; k++) {
+    const Dd64 f = dd64_from(d[k] * (mult(k) / (long double)n));
+    for (int j = 0, i = 0; j <= h; j++) {
+      r[j] = dd64_add(r[j], dd64_mul(f, cs[(size_t)i]));
+      i += k;
+      if (i >= n) i -= n;
     }
-    r[j] = a;
-    kmax = std::max(kmax, fabs(a.h));
-    ksum += mult(j) * fabs(a.h);
+  }
+  double kmax = 0.0, ksum = 0.0;
+  for (int j = 0; j <= h; j++) {
+    kmax = std::max(kmax, fabs(r[j].h));
+    ksum += mult(j) * fabs(r[j].h);
   }
   // |K_0| <= 2^11 - 2 (exact in FP16 after the correction of its sum), sum |K_0| <= 2^13
   int p = 13;
