@@ -309,7 +309,8 @@ pft_status pft_batch_get_fields(pft_batch* b, int i, void* wp, void* wm, pft_mem
 /* `updates` field updates of every member: solve (Eqs. 3-5, 8, 13) then the field
  * step of Eq. 9 -- explicit Euler with `lam` for SCFT members, Euler-Maruyama with
  * `dt` and the library's Philox noise for CL members.  GRAPHED captures one update of
- * the whole batch as a CUDA graph (recaptured when lam or dt change) and replays it.
+ * the whole batch as a CUDA graph and replays it; the first update, and the first after
+ * lam, dt or a plan change, is enqueued launch by launch and the graph made behind it.
  * Asynchronous on the batch stream.  Error: PFT_ERR_STATE if a member has no fields. */
 pft_status pft_batch_run(pft_batch* b, int updates, double lam, double dt, pft_batch_mode mode);
 

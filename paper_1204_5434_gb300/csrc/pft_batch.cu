@@ -109,14 +109,15 @@ constexpr int kMarchLanes = 6, kFinishLanes = 4;
 constexpr double kGroupBytes = 16e6;
 constexpr double kGroupSlices = 6.0;  // a member's slices: both fields, both newest slices, B_A, B_B
 
-std::vector<BatchGroup> batch_groups(const pft_batch* b) {
+// whole: one group a class.
+std::vector<BatchGroup> batch_groups(const pft_batch* b, bool whole) {
   std::vector<BatchGroup> out;
   for (size_t i = 0; i < b->classes.size(); i++) {
     const BatchClass& c = b->classes[i];
     const pft::CtxData& d = b->inst[c.members[0]]->d;
     const double slice = (double)d.M * (d.prec == PFT_FP64 ? 8 : 4) * (d.kind == PFT_SCFT_REAL ? 1 : 2);
     const int K = (int)c.members.size();
-    const int per = std::max(1, (int)(kGroupBytes / (kGroupSlices * slice)));
+    const int per = whole ? K : std::max(1, (int)(kGroupBytes / (kGroupSlices * slice)));
     const int ng = (K + per - 1) / per;
     for (int q = 0; q < ng; q++) {
       BatchGroup g{(int)i, (int)((long long)K * q / ng), (int)((long long)K * (q + 1) / ng), 0.0};
@@ -323,8 +324,11 @@ pft_status record_class_solve(pft_batch* b, BatchClass& c, long long* launches) 
 
 // One field update of every instance: the groups of members spread over the march streams (each
 // forked from and joined back into b->stream), each member's quadrature and field step on a finish
-// stream once its own marches are done, then the step counters on b->stream.
-pft_status record_update(pft_batch* b, double lam, double dt) {
+// stream once its own marches are done, then the step counters on b->stream.  `direct`: enqueued,
+// not captured; then whole classes (half the launches, 2 us of the host each) with the finishes on
+// the march streams (streams beyond the device's eight hardware queues share one and wait for one
+// another).
+pft_status record_update(pft_batch* b, double lam, double dt, bool direct) {
   long long launches = 0;
   cudaError_t e = cudaEventRecord(b->fork, b->stream);
   for (auto& l : b->march) {
@@ -335,19 +339,23 @@ pft_status record_update(pft_batch* b, double lam, double dt) {
     if (e == cudaSuccess) e = cudaStreamWaitEvent(l.stream, b->fork, 0);
   if (e != cudaSuccess) return bcuda(e, "batch fork");
   int nf = 0;
-  for (const BatchGroup& g : batch_groups(b)) {
+  pft_status st = PFT_OK;
+  for (const BatchGroup& g : batch_groups(b, direct)) {
     BatchClass& c = b->classes[g.cls];
     BatchLane& l = *std::min_element(b->march.begin(), b->march.end(),
                                      [](const BatchLane& x, const BatchLane& y) { return x.load < y.load; });
     l.load += g.work;
     for (int k = g.k0; k < g.k1; k++) b->inst[c.members[k]]->d.stream = l.stream;
-    pft_status s = record_marches(b, c, g.k0, g.k1, &launches, l.stream, [&](int k) {
+    st = record_marches(b, c, g.k0, g.k1, &launches, l.stream, [&](int k) {
       pft_ctx* x = b->inst[c.members[k]];
-      BatchLane& f = b->finish[nf++ % b->finish.size()];
-      cudaError_t e = cudaEventRecord(l.event, l.stream);
-      if (e == cudaSuccess) e = cudaStreamWaitEvent(f.stream, l.event, 0);
-      if (e != cudaSuccess) return bcuda(e, "member fork");
-      x->d.stream = f.stream;
+      cudaError_t e = cudaSuccess;
+      if (!direct) {
+        BatchLane& f = b->finish[nf++ % b->finish.size()];
+        e = cudaEventRecord(l.event, l.stream);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(f.stream, l.event, 0);
+        if (e != cudaSuccess) return bcuda(e, "member fork");
+        x->d.stream = f.stream;
+      }
       pft_status s = record_finish(b, c, k, &launches);
       if (s != PFT_OK) return s;
       const bool scft = (x->d.kind == PFT_SCFT_REAL);
@@ -357,13 +365,14 @@ pft_status record_update(pft_batch* b, double lam, double dt) {
       return e == cudaSuccess ? PFT_OK : bcuda(e, "batched field step");
     });
     for (int k = g.k0; k < g.k1; k++) b->inst[c.members[k]]->d.stream = b->stream;
-    if (s != PFT_OK) return s;
+    if (st != PFT_OK) break;
   }
-  for (auto* lanes : {&b->march, &b->finish})
+  for (auto* lanes : {&b->march, &b->finish})  // after an error too: what was launched is joined
     for (auto& l : *lanes) {
       if (e == cudaSuccess) e = cudaEventRecord(l.event, l.stream);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, l.event, 0);
     }
+  if (st != PFT_OK) return st;
   if (e != cudaSuccess) return bcuda(e, "batch join");
   const int n = (int)b->inst.size();
   k_batch_increment<<<(n + 255) / 256, 256, 0, b->stream>>>(b->d_steps, n);
@@ -371,6 +380,26 @@ pft_status record_update(pft_batch* b, double lam, double dt) {
   e = cudaGetLastError();
   if (e != cudaSuccess) return bcuda(e, "batched step counter");
   b->launches = launches;
+  return PFT_OK;
+}
+
+// The graph of one update.
+pft_status make_graph(pft_batch* b, double lam, double dt) {
+  cudaGraph_t g = nullptr;
+  cudaError_t e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
+  if (e != cudaSuccess) return bcuda(e, "batch capture");
+  pft_status s = record_update(b, lam, dt, false);
+  e = cudaStreamEndCapture(b->stream, &g);
+  if (s != PFT_OK) {
+    if (g) cudaGraphDestroy(g);
+    return s;
+  }
+  if (e != cudaSuccess) return bcuda(e, "batch capture end");
+  e = cudaGraphInstantiate(&b->graph, g, 0);
+  cudaGraphDestroy(g);
+  if (e != cudaSuccess) return bcuda(e, "batch graph instantiate");
+  b->g_lam = lam;
+  b->g_dt = dt;
   return PFT_OK;
 }
 
@@ -545,35 +574,36 @@ pft_status pft_batch_run(pft_batch* b, int updates, double lam, double dt, pft_b
     pft_status s = prepare_pairs(b, c);
     if (s != PFT_OK) return s;
   }
+  int run = 0;  // updates enqueued
+  pft_status s = PFT_OK;
   if (mode == PFT_BATCH_GRAPHED) {
     if (!b->graph || lam != b->g_lam || dt != b->g_dt) {
       if (b->graph) {
         cudaGraphExecDestroy(b->graph);
         b->graph = nullptr;
       }
+      // a stream that cannot be captured is refused before anything runs on it
       cudaGraph_t g = nullptr;
       cudaError_t e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
+      if (e == cudaSuccess) e = cudaStreamEndCapture(b->stream, &g);
       if (e != cudaSuccess) return bcuda(e, "batch capture");
-      pft_status s = record_update(b, lam, dt);
-      e = cudaStreamEndCapture(b->stream, &g);
-      if (s != PFT_OK) {
-        if (g) cudaGraphDestroy(g);
-        return s;
-      }
-      if (e != cudaSuccess) return bcuda(e, "batch capture end");
-      e = cudaGraphInstantiate(&b->graph, g, 0);
       cudaGraphDestroy(g);
-      if (e != cudaSuccess) return bcuda(e, "batch graph instantiate");
-      b->g_lam = lam;
-      b->g_dt = dt;
+      // The first update runs launch by launch, and while the GPU works on it the host makes the
+      // graph of the later ones (2.5 us a launch; 64 members of 32^3 to 64^3, 5064 launches: 13
+      // ms), which a first update, or one with another lam or dt, would else wait for.
+      if (updates > 0) {
+        if ((s = record_update(b, lam, dt, true)) != PFT_OK) return s;
+        run = 1;
+      }
+      s = make_graph(b, lam, dt);
     }
-    for (int u = 0; u < updates; u++) {
+    for (; s == PFT_OK && run < updates; run++) {
       cudaError_t e = cudaGraphLaunch(b->graph, b->stream);
-      if (e != cudaSuccess) return bcuda(e, "batch graph launch");
+      if (e != cudaSuccess) s = bcuda(e, "batch graph launch");
     }
   } else if (mode == PFT_BATCH_PER_INSTANCE) {
     const int n = (int)b->inst.size();
-    for (int u = 0; u < updates; u++) {
+    for (; s == PFT_OK && run < updates; run++) {
       for (pft_ctx* x : b->inst) {
         const bool scft = (x->d.kind == PFT_SCFT_REAL);
         cudaError_t e = x->eng->enqueue_solve(x->d);
@@ -590,11 +620,11 @@ pft_status pft_batch_run(pft_batch* b, int updates, double lam, double dt, pft_b
     return bfail(PFT_ERR_ARG, "unknown batch mode");
   }
   for (pft_ctx* x : b->inst) {
-    x->d.step += updates;
+    x->d.step += run;
     x->d.solved = false;
-    if (updates > 0) x->have_obs = true;
+    if (run > 0) x->have_obs = true;
   }
-  return PFT_OK;
+  return s;
 }
 
 pft_status pft_batch_autotune(pft_batch* b) {

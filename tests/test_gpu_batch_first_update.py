@@ -1,0 +1,89 @@
+"""The first update of a batch, and the first with another time step, before its graph exists:
+the same results as the later ones, and the host's work on the graph behind the GPU's on the
+update.  48 uneven systems take some 20 ms an update and their graph some 10 ms of the host; an
+update that waits for its graph takes half as long again as one that does not, so a quarter is
+allowed."""
+import time
+
+import numpy as np
+import pytest
+
+from paper_1204_5434_gb300 import pft
+
+pytestmark = pytest.mark.gpu
+SCFT, CL = pft.PFT_SCFT_REAL, pft.PFT_CL_COMPLEX
+LAM, DT = 0.1, 0.01
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_1204_5434_gb300 import build
+    build.build()
+
+
+def _batch(descs, seed):
+    b = pft.pft_batch_create(descs, pft.PFT_FP32_MIXED)
+    rng = np.random.default_rng(seed)
+    for i, d in enumerate(descs):
+        wp, wm = rng.normal(0, 0.1, d["n"]), rng.normal(0, 0.5, d["n"])
+        if d["kind"] == CL:
+            wp, wm = wp.astype(complex), wm.astype(complex)
+        pft.pft_batch_set_fields(b, i, wp, wm)
+    return b
+
+
+def _fields(b, descs):
+    out = []
+    for i, d in enumerate(descs):
+        dt = np.float64 if d["kind"] == SCFT else np.complex128
+        gp, gm = np.empty(d["n"], dt), np.empty(d["n"], dt)
+        pft.pft_batch_get_fields(b, i, gp, gm)
+        out.append(gp.tobytes() + gm.tobytes())
+    return out
+
+
+def _desc(n, ns, cl, i):
+    return dict(n=(n, n, n), L=(n / 8.0,) * 3, Ns=ns, fA=0.4, chiN=15.0, C=50.0 if cl else 1.0,
+                kind=CL if cl else SCFT, seed=70 + i)
+
+
+def test_same_results_however_the_updates_are_run():
+    """Five updates at once, one by one, with a dt that changes and comes back, and after a graph
+    made without an update: the same bits (the time step acts on the CL members alone)."""
+    descs = [_desc(n, ns, cl, i) for i, (n, ns, cl) in enumerate(
+        [(32, 9, True), (16, 4, True), (16, 12, False), (48, 5, False), (32, 1, True)])]
+    runs = [[(5, DT)], [(1, DT)] * 5, [(0, DT), (3, DT), (2, DT)],
+            [(2, DT), (1, 2 * DT), (2, DT)], [(1, DT), (1, DT), (1, 2 * DT), (1, DT), (1, DT)]]
+    out = []
+    for calls in runs:
+        b = _batch(descs, 5)
+        try:
+            for k, dt in calls:
+                pft.pft_batch_run(b, k, LAM, dt)
+            pft.pft_batch_synchronize(b)
+            out.append(_fields(b, descs))
+        finally:
+            pft.pft_batch_destroy(b)
+    assert out[0] == out[1] == out[2]
+    assert out[3] == out[4]
+    assert out[0] != out[3]
+
+
+def test_first_update_does_not_wait_for_its_graph():
+    descs = [_desc((32, 48, 64)[i % 3], (50, 100, 200)[(i // 3) % 3], i >= 24, i) for i in range(48)]
+    b = _batch(descs, 6)
+
+    def update(dt):
+        t = time.perf_counter()
+        pft.pft_batch_run(b, 1, LAM, dt)
+        pft.pft_batch_synchronize(b)
+        return 1e3 * (time.perf_counter() - t)
+
+    try:
+        update(DT)
+        steady = min(update(DT) for _ in range(6))
+        changed = min(update(DT * (1 + 0.01 * k)) for k in range(1, 7))
+        print(f"\n48 systems: {steady:.2f} ms an update, {changed:.2f} ms the first with another dt")
+        assert changed <= 1.25 * steady
+    finally:
+        pft.pft_batch_destroy(b)
