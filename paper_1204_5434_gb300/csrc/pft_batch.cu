@@ -109,10 +109,11 @@ constexpr int kMarchLanes = 6, kFinishLanes = 4;
 constexpr double kGroupBytes = 16e6;
 constexpr double kGroupSlices = 6.0;  // a member's slices: both fields, both newest slices, B_A, B_B
 
-// whole: one group a class.
-std::vector<BatchGroup> batch_groups(const pft_batch* b, bool whole) {
+// cls: one class (-1: all); whole: one group a class.
+std::vector<BatchGroup> batch_groups(const pft_batch* b, int cls, bool whole) {
   std::vector<BatchGroup> out;
   for (size_t i = 0; i < b->classes.size(); i++) {
+    if (cls >= 0 && (int)i != cls) continue;
     const BatchClass& c = b->classes[i];
     const pft::CtxData& d = b->inst[c.members[0]]->d;
     const double slice = (double)d.M * (d.prec == PFT_FP64 ? 8 : 4) * (d.kind == PFT_SCFT_REAL ? 1 : 2);
@@ -316,20 +317,14 @@ pft_status record_finish(pft_batch* b, const BatchClass& c, int k, long long* la
   return e == cudaSuccess ? PFT_OK : bcuda(e, "batched quadrature");
 }
 
-// A whole class on b->stream (the autotuner's unit).
-pft_status record_class_solve(pft_batch* b, BatchClass& c, long long* launches) {
-  return record_marches(b, c, 0, (int)c.members.size(), launches, b->stream,
-                        [&](int k) { return record_finish(b, c, k, launches); });
-}
-
-// One field update of every instance: the groups of members spread over the march streams (each
-// forked from and joined back into b->stream), each member's quadrature and field step on a finish
-// stream once its own marches are done, then the step counters on b->stream.  `direct`: enqueued,
+// The solves of class `cls` (-1: every instance): the groups of members spread over the march
+// streams (each forked from and joined back into b->stream), each member's quadrature, and what
+// after(member) records, on a finish stream once its own marches are done.  `direct`: enqueued,
 // not captured; then whole classes (half the launches, 2 us of the host each) with the finishes on
 // the march streams (streams beyond the device's eight hardware queues share one and wait for one
 // another).
-pft_status record_update(pft_batch* b, double lam, double dt, bool direct) {
-  long long launches = 0;
+template <typename F>
+pft_status record_solves(pft_batch* b, int cls, bool direct, long long* launches, F after) {
   cudaError_t e = cudaEventRecord(b->fork, b->stream);
   for (auto& l : b->march) {
     if (e == cudaSuccess) e = cudaStreamWaitEvent(l.stream, b->fork, 0);
@@ -340,13 +335,13 @@ pft_status record_update(pft_batch* b, double lam, double dt, bool direct) {
   if (e != cudaSuccess) return bcuda(e, "batch fork");
   int nf = 0;
   pft_status st = PFT_OK;
-  for (const BatchGroup& g : batch_groups(b, direct)) {
+  for (const BatchGroup& g : batch_groups(b, cls, direct)) {
     BatchClass& c = b->classes[g.cls];
     BatchLane& l = *std::min_element(b->march.begin(), b->march.end(),
                                      [](const BatchLane& x, const BatchLane& y) { return x.load < y.load; });
     l.load += g.work;
     for (int k = g.k0; k < g.k1; k++) b->inst[c.members[k]]->d.stream = l.stream;
-    st = record_marches(b, c, g.k0, g.k1, &launches, l.stream, [&](int k) {
+    st = record_marches(b, c, g.k0, g.k1, launches, l.stream, [&](int k) {
       pft_ctx* x = b->inst[c.members[k]];
       cudaError_t e = cudaSuccess;
       if (!direct) {
@@ -356,12 +351,9 @@ pft_status record_update(pft_batch* b, double lam, double dt, bool direct) {
         if (e != cudaSuccess) return bcuda(e, "member fork");
         x->d.stream = f.stream;
       }
-      pft_status s = record_finish(b, c, k, &launches);
+      pft_status s = record_finish(b, c, k, launches);
       if (s != PFT_OK) return s;
-      const bool scft = (x->d.kind == PFT_SCFT_REAL);
-      e = x->eng->field_step(x->d, scft ? PFT_STEP_SCFT_EULER : PFT_STEP_CL_EULER_MARUYAMA, scft ? lam : dt, nullptr,
-                             nullptr);
-      launches += 2;
+      e = after(x);
       return e == cudaSuccess ? PFT_OK : bcuda(e, "batched field step");
     });
     for (int k = g.k0; k < g.k1; k++) b->inst[c.members[k]]->d.stream = b->stream;
@@ -373,34 +365,91 @@ pft_status record_update(pft_batch* b, double lam, double dt, bool direct) {
       if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, l.event, 0);
     }
   if (st != PFT_OK) return st;
-  if (e != cudaSuccess) return bcuda(e, "batch join");
+  return e == cudaSuccess ? PFT_OK : bcuda(e, "batch join");
+}
+
+// One field update of every instance: the solves, each with its field step, then the step
+// counters on b->stream.
+pft_status record_update(pft_batch* b, double lam, double dt, bool direct) {
+  long long launches = 0;
+  pft_status s = record_solves(b, -1, direct, &launches, [&](pft_ctx* x) {
+    const bool scft = (x->d.kind == PFT_SCFT_REAL);
+    launches += 2;
+    return x->eng->field_step(x->d, scft ? PFT_STEP_SCFT_EULER : PFT_STEP_CL_EULER_MARUYAMA, scft ? lam : dt, nullptr,
+                              nullptr);
+  });
+  if (s != PFT_OK) return s;
   const int n = (int)b->inst.size();
   k_batch_increment<<<(n + 255) / 256, 256, 0, b->stream>>>(b->d_steps, n);
   launches += 1;
-  e = cudaGetLastError();
+  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return bcuda(e, "batched step counter");
   b->launches = launches;
   return PFT_OK;
 }
 
-// The graph of one update.
-pft_status make_graph(pft_batch* b, double lam, double dt) {
+// What record() enqueues from and to b->stream, as a graph.
+template <typename F> pft_status capture(pft_batch* b, cudaGraphExec_t* out, F record) {
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return bcuda(e, "batch capture");
-  pft_status s = record_update(b, lam, dt, false);
+  pft_status s = record();
   e = cudaStreamEndCapture(b->stream, &g);
   if (s != PFT_OK) {
     if (g) cudaGraphDestroy(g);
     return s;
   }
   if (e != cudaSuccess) return bcuda(e, "batch capture end");
-  e = cudaGraphInstantiate(&b->graph, g, 0);
+  e = cudaGraphInstantiate(out, g, 0);
   cudaGraphDestroy(g);
-  if (e != cudaSuccess) return bcuda(e, "batch graph instantiate");
+  return e == cudaSuccess ? PFT_OK : bcuda(e, "batch graph instantiate");
+}
+
+// The graph of one update.
+pft_status make_graph(pft_batch* b, double lam, double dt) {
+  pft_status s = capture(b, &b->graph, [&] { return record_update(b, lam, dt, false); });
+  if (s != PFT_OK) return s;
   b->g_lam = lam;
   b->g_dt = dt;
   return PFT_OK;
+}
+
+// Can the batch stream be captured (a legacy stream, or one being captured, cannot)?
+cudaError_t try_capture(pft_batch* b) {
+  cudaGraph_t g = nullptr;
+  cudaError_t e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
+  if (e == cudaSuccess) e = cudaStreamEndCapture(b->stream, &g);
+  if (e == cudaSuccess) e = cudaGraphDestroy(g);
+  return e;
+}
+
+// Time of one solve of class `cls` under its plan, as the update runs it: its groups on the march
+// streams, captured (launch by launch where the stream allows no capture).  The class whole on one
+// stream orders the plans otherwise: 200 members of 16^3, complex FP64, plans 0 / 3, ms: 40.4 / 41.4
+// against 31.7 / 26.1 in the update.
+pft_status time_class(pft_batch* b, int cls, cudaEvent_t e0, cudaEvent_t e1, float* ms) {
+  long long n = 0;
+  cudaGraphExec_t graph = nullptr;
+  auto solves = [&](bool direct) {
+    return record_solves(b, cls, direct, &n, [](pft_ctx*) { return cudaSuccess; });
+  };
+  const bool direct = try_capture(b) != cudaSuccess;
+  if (direct) (void)cudaGetLastError();
+  pft_status s = direct ? PFT_OK : capture(b, &graph, [&] { return solves(false); });
+  cudaError_t e = cudaSuccess;
+  auto solve = [&] {
+    if (direct) s = solves(true);
+    else e = cudaGraphLaunch(graph, b->stream);
+  };
+  if (s == PFT_OK) solve();  // warm-up
+  if (s == PFT_OK && e == cudaSuccess) e = cudaEventRecord(e0, b->stream);
+  if (s == PFT_OK && e == cudaSuccess) solve();
+  if (s == PFT_OK && e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
+  if (s == PFT_OK && e == cudaSuccess) e = cudaEventSynchronize(e1);
+  if (s == PFT_OK && e == cudaSuccess) e = cudaEventElapsedTime(ms, e0, e1);
+  if (graph) cudaGraphExecDestroy(graph);
+  if (s != PFT_OK) return s;
+  return e == cudaSuccess ? PFT_OK : bcuda(e, "autotune timing");
 }
 
 }  // namespace
@@ -583,11 +632,8 @@ pft_status pft_batch_run(pft_batch* b, int updates, double lam, double dt, pft_b
         b->graph = nullptr;
       }
       // a stream that cannot be captured is refused before anything runs on it
-      cudaGraph_t g = nullptr;
-      cudaError_t e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
-      if (e == cudaSuccess) e = cudaStreamEndCapture(b->stream, &g);
+      const cudaError_t e = try_capture(b);
       if (e != cudaSuccess) return bcuda(e, "batch capture");
-      cudaGraphDestroy(g);
       // The first update runs launch by launch, and while the GPU works on it the host makes the
       // graph of the later ones (2.5 us a launch; 64 members of 32^3 to 64^3, 5064 launches: 13
       // ms), which a first update, or one with another lam or dt, would else wait for.
@@ -645,18 +691,8 @@ pft_status pft_batch_autotune(pft_batch* b) {
       if (!eng->batch_plan_ok(c.g, plan)) continue;
       c.plan = plan;
       if (plan >= 1 && (st = prepare_pairs(b, c)) != PFT_OK) break;
-      long long n = 0;
-      if ((st = record_class_solve(b, c, &n)) != PFT_OK) break;  // warm-up
-      cudaEventRecord(e0, b->stream);
-      if ((st = record_class_solve(b, c, &n)) != PFT_OK) break;
-      cudaEventRecord(e1, b->stream);
-      e = cudaEventSynchronize(e1);
       float ms = 0.f;
-      if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-      if (e != cudaSuccess) {
-        st = bcuda(e, "autotune timing");
-        break;
-      }
+      if ((st = time_class(b, (int)(&c - b->classes.data()), e0, e1, &ms)) != PFT_OK) break;
       c.tuned_ms[pi] = ms;
       if (best < 0.f || ms < best) {
         best = ms;
