@@ -24,7 +24,7 @@
  *     re, im).  All API-facing arrays are float64 / complex128 in either precision.
  *   - PFT_FP64 runs every step to double accuracy: fields, propagators, Boltzmann factors and
  *     sums are doubles; the pencil march's convolutions along axes of 16, 32, 48, 64, 96 and
- *     128 points are exact sums of integer products on the tensor cores (values scaled by
+ *     128 points are sums of integer products on the tensor cores (values scaled by
  *     the largest of their line, the rounding 2^-54 of it or less), rounded once to double.
  *     PFT_FP32_MIXED runs the propagators, FFTs
  *     and Boltzmann factors in float (the integrand q*qd of the contour quadrature is

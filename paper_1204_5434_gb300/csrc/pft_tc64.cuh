@@ -11,11 +11,19 @@
 //      rounding of every K_j is chosen so that the sum of K_0 is 2^p and the sum of every other
 //      K_j is zero: what the products left out below do to the mean of a line vanishes.
 // Level l collects the products X_i K_j with i + j = l in one FP32 accumulator of the tensor
-// core: integers below 2^24 in sum, hence exact in any order of addition.  Levels 0 to 5 (21
-// products) are added up in 64-bit integers, level 5 with X_0 K_6 (K_6 stored 2^-9 smaller: an
-// error of the kernel acts at every step, and its seventh digit keeps that below 1e-18 a step);
-// the other products of level 6 are 2^-57 of S.  The sum is rounded once, to FP64.  Propagator slices against the FP64 oracle: 2e-16 to 8e-16 relative
-// (the FFT pair in FP64: the same or larger; the products with the Boltzmann factors set it).
+// core: integers, exact in any order of addition while their sums stay below 2^24.  Whatever the
+// digits, that holds up to 64 points on levels 0 to 4, at 128 points on levels 0 to 2 and at 96,
+// for kernels narrower than half the box, on 0 to 3.  Beyond it is not a bound: were every digit to
+// line up with the kernel's signs, level 3 would reach 1.5 and level 5 2.2 times 2^24 (kernels of
+// 0.02 to 400 grid cells), and an addition would round by two units, 2^-48 of S on level 3, 2^-57 on
+// 4.  Digits without that order reach 0.3.  Level 5 holds X_0 K_6 too, K_6 stored 2^-9 smaller (an error of the kernel acts at
+// every step, and its seventh digit keeps that below 1e-18 a step): fractions, rounded below 2^-60
+// of S.  Levels 0 to 5 (22 products) are added up in 64-bit integers; the other products of
+// level 6 are 2^-57 of S.  The sum is rounded once, to FP64.  Propagator slices against the FP64
+// oracle: 2e-16 to 8e-16 relative (the FFT pair in FP64: the same or larger; the products with
+// the Boltzmann factors set it).  128^3, Ns 100, phi against an extended-precision march: 2.3e-16, the
+// FFT march 2.3e-15 (an FP64 reference whose diffusion factor is one rounded exponential is itself
+// 1.6e-14 off).
 //
 // One CTA holds one tile: G warpgroups of 128 threads (thread = line) and one more warp that
 // issues the products, level by level into a ring of NB accumulators, while the warpgroups
@@ -117,7 +125,7 @@ inline const std::vector<Dd64>& tc64_cosines(int n) {
   }
 }
 
-// The table of one axis: the header {int p, growth bits, float sum |kern|}, then the blocks of K_0 .. K_6: block s
+// The table of one axis: the header {int p}, then the blocks of K_0 .. K_6: block s
 // of a digit holds kern[(8 (s - n/8 + 1) + r - e) mod n] at row r, element e.  d: the axis' factors exp(-k_a^2 ds) at k = 0 .. n/2.
 inline void tc64_build_table(int n, const long double* d, unsigned char* dst) {
   const int h = n / 2;
@@ -144,10 +152,6 @@ inline void tc64_build_table(int n, const long double* d, unsigned char* dst) {
   for (int j = 0; j <= h; j++) r[j] = {ldexp(r[j].h, p), ldexp(r[j].l, p)};
   memset(dst, 0, kTc64Head);
   memcpy(dst, &p, sizeof(p));
-  const int grow = ksum < 1.999 ? 1 : 2;  // the values of a convolution stay below 2^grow of its input's largest
-  memcpy(dst + 4, &grow, sizeof(grow));
-  const float ks = (float)(ksum * 1.000001);
-  memcpy(dst + 8, &ks, sizeof(ks));
   const int nslot = 2 * (n / 8) - 1;
   std::vector<double> q((size_t)h + 1);
   std::vector<__half> q16((size_t)3 * n);  // the digit at distance j, over three periods
