@@ -1888,6 +1888,11 @@ class EngineT : public Engine {
     const size_t slice = (size_t)c.M * sizeof(T);
     cudaError_t e;
     if (!c.stepsg) {
+      // the table first: the spectra, which the solve can do without, must not take its room
+      const size_t table_b = (size_t)2 * c.Ns * sizeof(BatchStep);
+      void* table = nullptr;
+      e = cudaMalloc(&table, table_b);
+      if (e != cudaSuccess) return e;
       const size_t spec_b = (size_t)c.Ms * sizeof(Z);
       const int want = (int)std::min<size_t>(std::min(c.Ns, 32), std::max<size_t>(1, ((size_t)64 << 20) / (2 * spec_b)));
       if (want > 1 && !c.gspec) {
@@ -1918,11 +1923,13 @@ class EngineT : public Engine {
         for (int a = 0; a < 4; a++) u.tw[a] = v.tw[a] = t + c.tw_off[a];
         for (int a = 0; a < 3; a++) u.d[a] = v.d[a] = t + c.d_off[a];
       }
-      e = cudaMalloc(&c.stepsg, h.size() * sizeof(BatchStep));
-      if (e != cudaSuccess) return e;
-      c.bytes += h.size() * sizeof(BatchStep);
-      e = cudaMemcpy(c.stepsg, h.data(), h.size() * sizeof(BatchStep), cudaMemcpyHostToDevice);
-      if (e != cudaSuccess) return e;
+      e = cudaMemcpy(table, h.data(), table_b, cudaMemcpyHostToDevice);
+      if (e != cudaSuccess) {
+        cudaFree(table);
+        return e;
+      }
+      c.stepsg = table;
+      c.bytes += table_b;
     }
     BatchGeom g;
     for (int a = 0; a < 3; a++) g.n[a] = c.n[a];
