@@ -233,17 +233,20 @@ __device__ __forceinline__ void tc64_to_double(const long long (&t)[K], int eb, 
   }
 }
 // FP64 in the digits' form: X, the integer nearest x in units of 2^(eL - 1076) (eL the biased
-// exponent of the line's largest value, at least kTc64MinExp), plus the digits' biases, above 8
-// bits of no meaning: digit i of X plus its bias is at bit 8 + 9 (5 - i).  The biases, 256 (512
-// for the leading digit), make all digits non-negative.  Ties go to even: values of a few bits
-// below the unit meet them half of the time, and a fixed direction would shift every step's mean.
-constexpr int kTc64MinExp = 80;  // a line below 2^-943 counts as 2^-943
+// exponent of the line's largest value, at least 1), plus the digits' biases, above 8 bits of no
+// meaning: digit i of X plus its bias is at bit 8 + 9 (5 - i).  The biases, 256 (512 for the leading
+// digit), make all digits non-negative.  Ties go to even: values of a few bits below the unit meet
+// them half of the time, and a fixed direction would shift every step's mean.  Lines down to
+// the smallest subnormal keep their digits (0.3 to 1.4 % of a march for the two operations; a
+// branch that lifts small lines cost 1 to 3 %).
 constexpr unsigned long long kTc64Bias =
     256ull * (1ull + (1ull << 9) + (1ull << 18) + (1ull << 27) + (1ull << 36)) + (512ull << 45);
 __device__ __forceinline__ unsigned long long tc64_digits(double x, int eL) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const int sh = eL + 2 - (int)((hi >> 20) & 0x7ffu);  // 2 and more; a zero or subnormal: 64 and more
-  const unsigned mh = __funnelshift_l(lo, (hi & 0xfffffu) | 0x100000u, 11), ml = lo << 11;  // leading bit 63
+  // subnormals and zeros: no leading one, and the exponent of the smallest normal value
+  const unsigned ha = hi & 0x7fffffffu;
+  const int sh = eL + 2 - (int)(max(ha, 0x100000u) >> 20);  // 2 and more
+  const unsigned mh = __funnelshift_l(lo, min(ha, (hi & 0xfffffu) | 0x100000u), 11), ml = lo << 11;  // leading bit 63
   const bool far = sh >= 32;
   const unsigned a = far ? mh : ml, b = far ? 0u : mh;
   const int s5 = far ? sh - 32 : sh;
@@ -423,7 +426,7 @@ __device__ __forceinline__ void tc64_lines(const BatchStep& s, int nlines, int c
 #pragma unroll
     for (int w = 0; w < G; w++) eL = max(eL, lexp[w * 128 + m]);
     const bool bad = eL == 0x7ff;  // an infinity or a NaN: the line becomes NaN
-    eL = max(eL, kTc64MinExp);
+    eL = max(eL, 1);  // (subnormal lines: their unit is a subnormal's)
     set_range(eL, bad);
 #pragma unroll
     for (int j = 0; j < PPT / 8; j++) {
