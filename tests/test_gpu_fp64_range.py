@@ -77,6 +77,18 @@ def _check(n, L, Ns, fA, kind, streams, wp, wm):
     assert eQ <= 1e-12 and ephi <= 1e-10 and eq <= 1e-12
 
 
+@pytest.mark.parametrize("n,kind", [((96, 16, 48), SCFT), ((16, 64, 64), CL), ((32, 96, 128), CL), ((96, 128, 16), CL),
+                                    ((128, 48, 96), SCFT), ((128, 32, 16), CL)])
+def test_long_lines_on_every_axis(n, kind):
+    """96 and 128 points on each axis, and complex lines of 16 on x, on grids without an axis on the
+    FFT kernels (the last one's x launch is too short for the tensor cores)."""
+    rng = np.random.default_rng(813)
+    wp, wm = rng.normal(0, 0.3, n), rng.normal(0, 1.0, n)
+    if kind == CL:
+        wp, wm = wp + 1j * rng.normal(0, 0.3, n), wm + 1j * rng.normal(0, 0.3, n)
+    _check(n, (5.0, 4.0, 6.0), 4, 0.4, kind, 1, wp, wm)
+
+
 LD = np.longdouble
 
 
