@@ -249,7 +249,9 @@ pft_status pft_adjoint(pft_ctx* ctx, const void* dL_dphiA, const void* dL_dphiB,
  *     at fixed grid values, from the bilinear contraction of the forward and
  *     conjugate spectra with d(exp(-k^2 ds))/dL_a over every contour step.
  *   dlnQ_dL[3] (host, may be NULL).
- * SCFT mode only (PFT_ERR_UNSUPPORTED in CL mode).  Runs one extra march. */
+ * SCFT mode only (PFT_ERR_UNSUPPORTED in CL mode).  The first box derivative of a context
+ * allocates its step table and up to 64 MB for the spectra of several steps (one step at a
+ * time without them).  Errors: PFT_ERR_OOM if the table cannot be had. */
 pft_status pft_gradients(pft_ctx* ctx, void* dH_dwp, void* dH_dwm, double dH_dL[3],
                          double dlnQ_dL[3], pft_mem where);
 
@@ -293,10 +295,9 @@ typedef struct pft_batch pft_batch;
 
 /* Create `count` independent systems (SCFT and CL mixed; grid sizes up to 64 per axis
  * from 4,6,8,12,16,24,32,48,64; any Ns and fA) in one precision.  Members with equal
- * field kind and grid form a class; one field update of the whole batch runs each
- * contour step of each class as five batched launches over the members still
- * marching (members of a class sorted by Ns), then every member's reductions and
- * field update.  stream: cudaStream_t or NULL (the batch creates one).
+ * field kind and grid form a class, sorted by Ns; its members march in groups that share
+ * the launches of a contour step (one or two in the default plans) over those still
+ * marching, each member's reductions and field update following its own marches.  stream: cudaStream_t or NULL (the batch creates one).
  * Errors: PFT_ERR_ARG, PFT_ERR_SHAPE, PFT_ERR_OOM, PFT_ERR_CUDA. */
 pft_status pft_batch_create(pft_batch** out, int count, const pft_instance_desc* descs,
                             pft_precision precision, void* stream);

@@ -85,7 +85,7 @@ struct pft_batch {
   bool own_stream = false;
   std::vector<BatchClass> classes;
   unsigned long long* d_steps = nullptr;
-  int* d_err = nullptr;  // error word of the bounded waits in the separable plane kernel
+  int* d_err = nullptr;  // error word of the kernels' bounded waits
   cudaEvent_t fork = nullptr;
   std::vector<BatchLane> march, finish;
   cudaGraphExec_t graph = nullptr;
@@ -101,10 +101,12 @@ namespace {
 // each launch found the last one's field evicted from the 129 MB L2, and the quadratures (a
 // member's own history from DRAM, a few small launches) came one after the other at the classes'
 // ends.  Groups of at most 16 MB on six streams stay in L2 together, and a member's quadrature and
-// field step run beside the other groups' marches.  Measured, ms an update with fields in and out,
-// whole classes -> groups: 16 members 6.98 -> 6.91, 32 10.4 -> 10.4, 48 22.2 -> 20.4, 64 27.3 ->
-// 25.4, 128 53.7 -> 50.8; fewer streams lose where there are few members (16 members on four
-// streams of 32 MB 8.8), larger groups gain less (64 members, six streams: 32 MB 27.6, 64 MB 28.6).
+// field step run beside the other groups' marches.  Measured, ms an update without the fields'
+// copies, one group a class / 64 MB / 32 MB / 16 MB: FP32, 64 members 23.3 / 22.9 / 23.0 / 21.9, 24
+// members 10.2 / 10.1 / 9.8 / 10.0, 16 members 5.4 / 5.5 / 5.5 / 5.3, 8 members 3.2 / 3.3 / 3.3 / 3.3;
+// FP64 (a 64^3 complex member is 25 MB, a group of its own), 24 members 53.8 / 54.7 / 51.5 / 50.5, 16
+// members 24.2 / 24.3 / 24.3 / 23.5, 8 members 9.1 / 9.1 / 9.1 / 9.2.  Fewer streams lose where there
+// are few members (16 members on four streams of 32 MB: 1.3 times as long).
 constexpr int kMarchLanes = 6, kFinishLanes = 4;
 constexpr double kGroupBytes = 16e6;
 constexpr double kGroupSlices = 6.0;  // a member's slices: both fields, both newest slices, B_A, B_B
@@ -751,7 +753,7 @@ pft_status pft_batch_synchronize(pft_batch* b) {
   if (err != 0) {
     cudaMemsetAsync(b->d_err, 0, sizeof(int), b->stream);
     cudaStreamSynchronize(b->stream);
-    return bfail(PFT_ERR_TIMEOUT, "a bounded wait in a separable plane kernel ran out (the last updates are invalid)");
+    return bfail(PFT_ERR_TIMEOUT, "a bounded wait in a kernel of the last updates ran out (their results are invalid)");
   }
   return PFT_OK;
 }

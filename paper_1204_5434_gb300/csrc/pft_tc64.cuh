@@ -29,17 +29,19 @@
 // issues the products, level by level into a ring of NB accumulators, while the warpgroups
 // read the levels before.  A line with an infinity or a NaN becomes NaN, as under the FFT.
 //
-// What bounds it: the integer pipe (64 operations a cycle and SM; ncu: busy throughout) beside the
-// products.  A 64-point tile of 128 lines takes 15,000 cycles without and 37,000 with the Boltzmann
-// products: 3,800 for the products of a convolution (2,800 at the tensor core's rate), 4,400 for the
-// digits, 4,200 for each conversion back, 8,200 for two FP64 multiplications by B, 2,000 each to
-// load and to store.  The FFT pair needs about 26 FP64 operations a point and convolution, 13
-// cycles an SM, this 1.8 to 4.  At 128 points the 17 warps' cap of 96 registers costs spills too
-// (ptxas: 648 bytes stored a thread in the fused z kernel, 628 in x, 64 in y; complex fields 316,
-// 156, 64; at most 152 at 96 points and 44 below).
+// What bounds it: the chain of a tile's phases, which follow one another on 17 warps with one tile an
+// SM; no pipe is full (ncu, real fields, y kernel / fused x kernel: integer pipe 37 / 32 %, tensor
+// pipe 16 / 13 %, FP64 pipe 0 / 19 % at 64 points; 33 / 25, 28 / 21 and 0 / 15 % at 128, where the
+// fused kernels also wait for their instructions).  A 64-point tile of 128 lines takes 15,000 cycles
+// without and 37,000 with the Boltzmann products: 3,800 for the products of a convolution (2,800
+// at the tensor core's rate), 4,400 for the digits, 4,200 for each conversion back, 8,200 for two
+// FP64 multiplications by B, 2,000 each to load and to store.  The FFT pair needs about 26 FP64
+// operations a point and convolution, 13 cycles an SM, this 1.8 to 4.  At 128 points the 17 warps'
+// cap of 96 registers costs spills too (ptxas, bytes stored a thread: 648 in the fused z kernel, 628
+// in x, 88 in y; complex fields 276, 236, 88; at most 120 at 96 points and 12 at 64).
 // Measured, one field update with fields in and out, FFT pair -> this (ms): 32^3 real, Ns 64, 2.49 ->
-// 1.32; 64^3 real, Ns 100, 6.59 -> 3.39, complex 12.26 -> 5.04; 128^3 real 50.9 -> 13.4, complex
-// 104.3 -> 37.0.
+// 1.33; 64^3 real, Ns 100, 6.59 -> 3.41, complex 12.26 -> 5.05; 128^3 real 50.9 -> 13.6, complex
+// 104.3 -> 37.3.
 // Tried: fields and factors in fixed point between the launches, one scale a slice (128^3 real 10.7
 // ms, 64^3 complex 3.3): lines and factors far below the slice's largest lose digits there, and
 // so does the block junction where the two blocks' largest factors lie apart (W- noise of 25, six
