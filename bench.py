@@ -38,15 +38,16 @@ WORK = wl.GYR128
 # conjugate step also reads the partner q and reads+writes an FP64 accumulator
 # (3e+f+2a).  Mean (5e+2f+2a)/2 with e=f=4, a=8 (FP32-mixed) or e=f=a=8 (FP64), real fields.
 BYTES_PER_UNIT = {"fp32": 22.0, "fp64": 36.0}
-# FP64: the denominator is the rate of the GB300 FP64 pipe, measured live (pft_fma_throughput, a
-# DFMA loop over every SM).  The march's convolutions run on the tensor cores as exact sums of
-# integer products, so the fraction passes 1; what bounds them is the integer ALU work of splitting
-# and summing, and the tensor rate is reported beside it (22 products of 2 n flops a point and axis).  Flops per unit: in the
-# usual 5 N log2 N convention a length-n complex transform of two paired real lines costs
-# 2.5 log2(n) flops per real point, so the separable march's forward and inverse transform
-# along each of the three axes cost 5 log2(M) per point and contour step -- the same count
-# as a real-to-half-spectrum 3D transform pair -- plus about 6 pointwise flops (two
-# Boltzmann multiplies, the diffusion multiplies, the quadrature update).
+# FP64: the march's convolutions run on the tensor cores as sums of integer products, 22 products of
+# 2 n flops a point and axis, and the fraction is theirs of the measured bf16 rate (the FP16 rate is
+# the same); what bounds them is the integer work of splitting and summing beside the products.
+# Beside it, as a comparison, the rate of the same transforms by FFT against the FP64 pipe
+# (pft_fma_throughput, a DFMA loop over every SM), which the march passes: in the usual 5 N log2 N
+# convention a length-n complex transform of two paired real lines costs 2.5 log2(n) flops per
+# real point, so the separable march's forward and inverse transform along each of the three axes
+# cost 5 log2(M) per point and contour step -- the same count as a real-to-half-spectrum 3D
+# transform pair -- plus about 6 pointwise flops (two Boltzmann multiplies, the diffusion
+# multiplies, the quadrature update).
 FP64_NOMINAL_TFLOPS = 1.25
 # DRAM traffic of one launch of the separable march (one contour step of one
 # propagator: a plane kernel or an x kernel in turn) on the FP32 128^3 path in steady state:
@@ -55,12 +56,12 @@ FP64_NOMINAL_TFLOPS = 1.25
 # previous launches left them (so each launch is charged with the write-backs its stores
 # cause).  Reads are nearly nil (the field and both factors stay in L2); the writes are the
 # q slices.  Valid only for the kernel sources it was taken on: null once any changes.
-TRAFFIC_FP32 = {"bytes_per_contour_step": 8601732.3,
+TRAFFIC_FP32 = {"bytes_per_contour_step": 8591104.0,
                 "sources": ("paper_1204_5434_gb300/csrc/pft_sep.cuh", "paper_1204_5434_gb300/csrc/pft_sepp.cuh",
                             "paper_1204_5434_gb300/csrc/pft_plane.cuh", "paper_1204_5434_gb300/csrc/pft_tma.cuh",
                             "paper_1204_5434_gb300/csrc/pft_batch.cuh", "paper_1204_5434_gb300/csrc/pft_passes.cuh",
                             "paper_1204_5434_gb300/csrc/pft_fft.cuh", "paper_1204_5434_gb300/csrc/pft_dd.cuh"),
-                "sha256": "622725bb0755c6269af6c5cbf8c16d2728d8ebe15014ce103e9939b980a6571d"}
+                "sha256": "7818dca885162163ef6a5eef168a692e8d82a1852a92f9b48ae6eeae9fd4586a"}
 
 
 def _traffic_fp32():
@@ -76,13 +77,13 @@ def fp64_flops_per_unit(M):
     return 5.0 * math.log2(M) + 6.0
 
 
-def _peaks():
+def _peaks(key="hbm_gbs", fallback=6800.0):
     p = os.path.join(ROOT, "MEASURED_PEAKS.json")
     if os.path.exists(p):
         with open(p) as f:
             d = json.load(f)
-        return float(d["hbm_gbs"]), "measured"
-    return 6800.0, "fallback"
+        return float(d[key]), "measured"
+    return fallback, "fallback"
 
 
 def _dist():
@@ -617,12 +618,13 @@ def run(args):
             tf = fpu * WORK.M / (step_ms * 1e-3) / 1e12
             dfma = pft.pft_fma_throughput(pft.PFT_FP64)
             mma = 22 * 2.0 * sum(WORK.n) * WORK.M / (step_ms * 1e-3) / 1e12
+            tc_peak, tc_src = _peaks("bf16_tflops", 1900.0)
             roof = {"bound": "alu", "kernel": "separable march on pencils: a y launch and an x or z launch per contour "
-                                              "step, convolutions on the tensor cores as exact integer products",
-                    "tensor_TFLOPs": mma,
-                    "achieved": tf, "peak": dfma, "unit": "TFLOP/s", "frac": tf / dfma,
-                    "peak_source": f"measured DFMA throughput of this GPU (pft_fma_throughput; nominal "
-                                   f"{FP64_NOMINAL_TFLOPS} TFLOP/s)",
+                                              "step, convolutions on the tensor cores as integer products",
+                    "achieved": mma, "peak": tc_peak, "unit": "TFLOP/s", "frac": mma / tc_peak,
+                    "peak_source": f"{tc_src} bf16_tflops (MEASURED_PEAKS.json); digit products, the integer work "
+                                   "beside them bounds the kernels",
+                    "fft_equivalent_TFLOPs": tf, "dfma_TFLOPs": dfma, "fft_equivalent_over_dfma": tf / dfma,
                     "flops_per_unit": fpu, "units_per_launch": WORK.M, "step_us": step_ms * 1e3,
                     "hbm_achieved_GBps": achieved, "hbm_frac": achieved / peak, "traffic": None}
         res[prec_name] = {

@@ -311,7 +311,8 @@ pft_status pft_batch_get_fields(pft_batch* b, int i, void* wp, void* wm, pft_mem
  * step of Eq. 9 -- explicit Euler with `lam` for SCFT members, Euler-Maruyama with
  * `dt` and the library's Philox noise for CL members.  GRAPHED captures one update of
  * the whole batch as a CUDA graph and replays it; the first update, and the first after
- * lam, dt or a plan change, is enqueued launch by launch and the graph made behind it.
+ * lam, dt or a plan change, is enqueued launch by launch and the graph made behind it (an
+ * error then leaves that update done and counted).
  * Asynchronous on the batch stream.  Error: PFT_ERR_STATE if a member has no fields. */
 pft_status pft_batch_run(pft_batch* b, int updates, double lam, double dt, pft_batch_mode mode);
 
