@@ -52,12 +52,13 @@ struct BatchClass {
 struct BatchLane {
   cudaStream_t stream = nullptr;
   cudaEvent_t event = nullptr;
-  double load = 0.0;  // work recorded on it
+  int load = 0;  // contour steps recorded on it
 };
 
-// Members k0 <= k < k1 of a class that march together.
+// Members k0 <= k < k1 of a class that march together; whole: all of them.
 struct BatchGroup {
   int cls, k0, k1;
+  bool whole;
   double work;
 };
 
@@ -96,35 +97,50 @@ struct pft_batch {
 
 namespace {
 
-// The update's streams and the working set of a group.  A class marched whole keeps every member's
-// field, factors and newest slices in turn: 64 members of 32^3 to 64^3 are some 300 MB, so that
-// each launch found the last one's field evicted from the 129 MB L2, and the quadratures (a
-// member's own history from DRAM, a few small launches) came one after the other at the classes'
-// ends.  Groups of at most 16 MB on six streams stay in L2 together, and a member's quadrature and
-// field step run beside the other groups' marches.  Measured, ms an update without the fields'
-// copies, one group a class / 64 MB / 32 MB / 16 MB: FP32, 64 members 23.3 / 22.9 / 23.0 / 21.9, 24
-// members 10.2 / 10.1 / 9.8 / 10.0, 16 members 5.4 / 5.5 / 5.5 / 5.3, 8 members 3.2 / 3.3 / 3.3 / 3.3;
-// FP64 (a 64^3 complex member is 25 MB, a group of its own), 24 members 53.8 / 54.7 / 51.5 / 50.5, 16
-// members 24.2 / 24.3 / 24.3 / 23.5, 8 members 9.1 / 9.1 / 9.1 / 9.2.  Fewer streams lose where there
-// are few members (16 members on four streams of 32 MB: 1.3 times as long).
-constexpr int kMarchLanes = 6, kFinishLanes = 4;
-constexpr double kGroupBytes = 16e6;
+// The update's streams and the working set of a group.  A march is a chain of dependent launches,
+// so the chains of different classes run beside one another, a march stream each (six at least, for
+// the groups of few classes), the next group going to the stream with the fewest steps so far.
+//
+// Groups: a class marched whole keeps every member's field, factors and newest slices in turn, and
+// where they pass the 129 MB L2 each launch finds the last one's field evicted; groups of at most
+// 16 MB on six streams stay in L2 together.  But groups are more chains of smaller launches: where
+// the whole batch nearly fits (three classes or more, together below 175 MB and none above 90) its
+// classes march whole.  ms an update of 32^3 to 64^3 members with fields in and out, one stream a
+// class and its finishes behind it / groups always / this rule: 15 members 6.9 / 9.0 / 6.8, 18 6.5 /
+// 7.3 / 6.5, 22 9.6 / 11.1 / 9.4, 38 16.7 / 15.5 / 15.6, 64 27.4 / 25.1 / 24.5; a total of 120, 150 or 200 MB
+// for 175 loses up to 4 % at 28 to 31 members or gives up to 7 % away at 35 to 39.  One class: 12
+// members of 64^3 (complex, 151 MB) 17.1 / 13.6 / 13.6; FP64, 24 members 144 / 50.5 / 51.4, 16 64.2 / 23.5 /
+// 23.9.
+//
+// Finishes: a member's quadrature and field step, a few small launches, on one of the march
+// stream's own finish streams, a group's as soon as its member is done, a whole class's when the
+// class is.  Streams shared by all classes held the early ones' finishes up behind the late ones':
+// 101 members in ten classes 4.0 one stream a class, 5.2 shared, 3.7 now; 200 of one class 28.7, 11.5, 7.5.
+constexpr int kMarchLanes = 6, kMaxMarchLanes = 24, kFinishLanes = 24;
+constexpr double kBatchBytes = 175e6, kClassBytes = 90e6, kGroupBytes = 16e6;
 constexpr double kGroupSlices = 6.0;  // a member's slices: both fields, both newest slices, B_A, B_B
+
+double member_bytes(const pft_batch* b, const BatchClass& c) {
+  const pft::CtxData& d = b->inst[c.members[0]]->d;
+  return kGroupSlices * (double)d.M * (d.prec == PFT_FP64 ? 8 : 4) * (d.kind == PFT_SCFT_REAL ? 1 : 2);
+}
 
 // cls: one class (-1: all); whole: one group a class.
 std::vector<BatchGroup> batch_groups(const pft_batch* b, int cls, bool whole) {
   std::vector<BatchGroup> out;
+  double total = 0.0;
+  for (const BatchClass& c : b->classes) total += member_bytes(b, c) * (double)c.members.size();
   for (size_t i = 0; i < b->classes.size(); i++) {
     if (cls >= 0 && (int)i != cls) continue;
     const BatchClass& c = b->classes[i];
-    const pft::CtxData& d = b->inst[c.members[0]]->d;
-    const double slice = (double)d.M * (d.prec == PFT_FP64 ? 8 : 4) * (d.kind == PFT_SCFT_REAL ? 1 : 2);
+    const double bytes = member_bytes(b, c);
     const int K = (int)c.members.size();
-    const int per = whole ? K : std::max(1, (int)(kGroupBytes / (kGroupSlices * slice)));
+    const bool all = whole || (b->classes.size() > 2 && total <= kBatchBytes && bytes * K <= kClassBytes);
+    const int per = all ? K : std::max(1, (int)(kGroupBytes / bytes));
     const int ng = (K + per - 1) / per;
     for (int q = 0; q < ng; q++) {
-      BatchGroup g{(int)i, (int)((long long)K * q / ng), (int)((long long)K * (q + 1) / ng), 0.0};
-      for (int k = g.k0; k < g.k1; k++) g.work += slice * b->inst[c.members[k]]->d.Ns;
+      BatchGroup g{(int)i, (int)((long long)K * q / ng), (int)((long long)K * (q + 1) / ng), all, 0.0};
+      for (int k = g.k0; k < g.k1; k++) g.work += bytes * b->inst[c.members[k]]->d.Ns;
       out.push_back(g);
     }
   }
@@ -321,33 +337,41 @@ pft_status record_finish(pft_batch* b, const BatchClass& c, int k, long long* la
 
 // The solves of class `cls` (-1: every instance): the groups of members spread over the march
 // streams (each forked from and joined back into b->stream), each member's quadrature, and what
-// after(member) records, on a finish stream once its own marches are done.  `direct`: enqueued,
-// not captured; then whole classes (half the launches, 2 us of the host each) with the finishes on
-// the march streams (streams beyond the device's eight hardware queues share one and wait for one
-// another).
+// after(member) records, on a finish stream of its march stream.  `direct`: enqueued, not captured;
+// then whole classes (half the launches, 2 us of the host each) on the march streams alone, the
+// finishes on those without a class (streams beyond the device's eight hardware queues share one
+// and wait for one another).
 template <typename F>
 pft_status record_solves(pft_batch* b, int cls, bool direct, long long* launches, F after) {
   cudaError_t e = cudaEventRecord(b->fork, b->stream);
   for (auto& l : b->march) {
     if (e == cudaSuccess) e = cudaStreamWaitEvent(l.stream, b->fork, 0);
-    l.load = 0.0;
+    l.load = 0;
   }
   for (auto& l : b->finish)
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(l.stream, b->fork, 0);
+    if (e == cudaSuccess && !direct) e = cudaStreamWaitEvent(l.stream, b->fork, 0);
   if (e != cudaSuccess) return bcuda(e, "batch fork");
-  int nf = 0;
+  const size_t nfin = b->finish.size() / b->march.size();  // finish streams of a march stream
+  size_t nf = 0;
+  const std::vector<BatchGroup> groups = batch_groups(b, cls, direct);
+  // direct: the groups take a march stream each, the finishes those that are left, if they are
+  // enough of them (100 members of 24^3 11.8 ms against 19.9 with the finishes behind the march)
+  size_t idle = b->march.size() > groups.size() ? b->march.size() - groups.size() : 0;
+  if (idle < 3) idle = 0;
   pft_status st = PFT_OK;
-  for (const BatchGroup& g : batch_groups(b, cls, direct)) {
+  for (const BatchGroup& g : groups) {
     BatchClass& c = b->classes[g.cls];
-    BatchLane& l = *std::min_element(b->march.begin(), b->march.end(),
-                                     [](const BatchLane& x, const BatchLane& y) { return x.load < y.load; });
-    l.load += g.work;
+    const size_t li = std::min_element(b->march.begin(), b->march.end(),
+                                       [](const BatchLane& x, const BatchLane& y) { return x.load < y.load; }) -
+                      b->march.begin();
+    BatchLane& l = b->march[li];
+    l.load += b->inst[c.members[g.k0]]->d.Ns;
     for (int k = g.k0; k < g.k1; k++) b->inst[c.members[k]]->d.stream = l.stream;
-    st = record_marches(b, c, g.k0, g.k1, launches, l.stream, [&](int k) {
+    auto finish = [&](int k) {
       pft_ctx* x = b->inst[c.members[k]];
       cudaError_t e = cudaSuccess;
-      if (!direct) {
-        BatchLane& f = b->finish[nf++ % b->finish.size()];
+      if (!direct || idle > 0) {
+        const BatchLane& f = direct ? b->march[groups.size() + nf++ % idle] : b->finish[li * nfin + nf++ % nfin];
         e = cudaEventRecord(l.event, l.stream);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(f.stream, l.event, 0);
         if (e != cudaSuccess) return bcuda(e, "member fork");
@@ -357,12 +381,16 @@ pft_status record_solves(pft_batch* b, int cls, bool direct, long long* launches
       if (s != PFT_OK) return s;
       e = after(x);
       return e == cudaSuccess ? PFT_OK : bcuda(e, "batched field step");
-    });
+    };
+    st = record_marches(b, c, g.k0, g.k1, launches, l.stream,
+                        [&](int k) { return g.whole ? PFT_OK : finish(k); });
+    for (int k = g.k0; k < g.k1 && st == PFT_OK && g.whole; k++) st = finish(k);
     for (int k = g.k0; k < g.k1; k++) b->inst[c.members[k]]->d.stream = b->stream;
     if (st != PFT_OK) break;
   }
   for (auto* lanes : {&b->march, &b->finish})  // after an error too: what was launched is joined
     for (auto& l : *lanes) {
+      if (direct && lanes == &b->finish) break;
       if (e == cudaSuccess) e = cudaEventRecord(l.event, l.stream);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, l.event, 0);
     }
@@ -509,17 +537,6 @@ pft_status pft_batch_create(pft_batch** out, int count, const pft_instance_desc*
     batch_free(b);
     return bcuda(e, "batch fork event");
   }
-  b->march.resize(kMarchLanes);
-  b->finish.resize(kFinishLanes);
-  for (auto* lanes : {&b->march, &b->finish})
-    for (auto& l : *lanes) {
-      if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&l.stream, cudaStreamNonBlocking);
-      if (e == cudaSuccess) e = cudaEventCreateWithFlags(&l.event, cudaEventDisableTiming);
-    }
-  if (e != cudaSuccess) {
-    batch_free(b);
-    return bcuda(e, "batch streams");
-  }
   e = cudaMalloc(&b->d_err, 4 * sizeof(int));
   if (e == cudaSuccess) e = cudaMemsetAsync(b->d_err, 0, 4 * sizeof(int), b->stream);
   if (e != cudaSuccess) {
@@ -554,6 +571,18 @@ pft_status pft_batch_create(pft_batch** out, int count, const pft_instance_desc*
       it = index.find(key);
     }
     b->classes[it->second].members.push_back(i);
+  }
+  const int lanes = std::min(count, std::min(kMaxMarchLanes, std::max(kMarchLanes, (int)b->classes.size())));
+  b->march.resize(lanes);
+  b->finish.resize((size_t)lanes * std::max(1, std::min(4, kFinishLanes / lanes)));
+  for (auto* v : {&b->march, &b->finish})
+    for (auto& l : *v) {
+      if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&l.stream, cudaStreamNonBlocking);
+      if (e == cudaSuccess) e = cudaEventCreateWithFlags(&l.event, cudaEventDisableTiming);
+    }
+  if (e != cudaSuccess) {
+    batch_free(b);
+    return bcuda(e, "batch streams");
   }
   for (auto& c : b->classes) {
     std::stable_sort(c.members.begin(), c.members.end(),
